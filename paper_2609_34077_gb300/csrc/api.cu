@@ -142,17 +142,28 @@ unsigned* device_error_word() {
   return static_cast<unsigned*>(p);
 }
 
-WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank) {
+WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank, bool no_tc) {
   WsLayout L{};
   L.lrank = lrank;
-  L.tc = dtype == MCFT_BF16 && T > 64 && d % 256 == 0 && w % 128 == 0;
+  const bool aligned = tc_aligned(d, w);
+  L.tc = dtype == MCFT_BF16 && T > 64 && !no_tc;
   L.decode = !L.tc && dtype == MCFT_BF16;
   L.ks = L.decode ? decode_ksplit(T) : 1;
-  L.pad = !L.tc ? 1
-          : g_tc_tiles.load() == MCFT_TC_TILES_CTA_PAIR && tc_pair_tiles(T, K, E, lrank) ? 256
-                                                                                       : 128;
+  const bool pair = L.tc && aligned && g_tc_tiles.load() == MCFT_TC_TILES_CTA_PAIR &&
+                    tc_pair_tiles(T, K, E, lrank);
+  // The 128-row tiles of gemm_tc.cu keep the layers whose contractions are long and whose experts
+  // average many rows; everything else runs with the weight rows on M (gemm_rows.cu). Whole passes,
+  // gemm_tc against gemm_rows: Mixtral shape at T = 4096 (1024 rows by T K / E) 1978 / 2028 us and at
+  // 8192 3760 / 3977, but 928 / 792 at 1500 (375 rows) and at 3000 (750) even, 1496 / 1519;
+  // DeepSeek-V2-Lite shape (contractions of 2048 and 1408) 641 / 540 at 4096, 2112 / 1908 at 16384
+  // (1536 rows). The choice must not depend on adapters: mcft_gate_grad reads the workspace of a
+  // forward without knowing whether it had any.
+  const bool big = aligned && d >= 4096 && w >= 4096 && size_t(T) * K >= size_t(768) * E;
+  L.rows = L.tc && !pair && !big;
+  L.split = aligned ? 1 : 2;
+  L.pad = pair ? 256 : L.tc && !L.rows ? 128 : 1;
   const int nseg = E + S;
-  L.mcap = T * K + S * T + (L.tc ? nseg * (L.pad - 1) : 0);
+  L.mcap = T * K + S * T + nseg * (L.pad - 1);
   size_t o = 0;
   L.hdr = o;  o = align256(o + sizeof(WsHeader));
   L.cnt = o;  o = align256(o + sizeof(int) * nseg);
@@ -404,7 +415,7 @@ struct LoraArgs {
 mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, const int32_t* idx,
                          const float* gate, const void* const* experts, const void* const* shared,
                          const LoraArgs* lora, void* y, void* workspace, size_t ws_bytes,
-                         cudaStream_t stream) {
+                         cudaStream_t stream, bool no_tc = false) {
   mcft_status st = check_desc(desc);
   if (st != MCFT_OK) return st;
   if (T < 0) return fail(MCFT_ERR_INVALID, "T = %d < 0", T);
@@ -418,7 +429,7 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     return fail(MCFT_ERR_INVALID, "x and y must be 16-byte aligned");
   const int E = desc->E, S = desc->n_shared, K = desc->K;
   const int lrank = lora ? lora->rank : 0;
-  const WsLayout L = ws_layout(desc->d, E, K, desc->w, S, desc->dtype, T, lrank);
+  const WsLayout L = ws_layout(desc->d, E, K, desc->w, S, desc->dtype, T, lrank, no_tc);
   if (ws_bytes < L.total)
     return fail(MCFT_ERR_INVALID, "workspace of %zu bytes < %zu needed", ws_bytes, L.total);
   for (int e = 0; e < E; ++e)
@@ -493,21 +504,28 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     la.K = desc->d;
     la.u = const_cast<float*>(fa.u13);
     la.ustride = 2 * lrank;
-    if (!L.tc) {  // the tcgen05 path projects the gathered rows instead, after the gather
+    la.scale = lora->scale;
+    la.split = L.split;
+    if (L.rows) {
+      e = launch_lora_down_tiles(la, 2 * lrank, L.mcap, num_sms(), stream);
+      if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
+    } else if (!L.tc) {  // the padded tiles project the gathered rows instead, after the gather
       e = launch_lora_down(la, desc->dtype, 2 * lrank, L.mcap, stream);
       if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
     }
   }
   auto ffn = [&](int stages) -> cudaError_t {
+    if (L.rows) return launch_ffn_rows(fa, ws + L.xp, L.mcap, num_sms(), stream, stages, L.split);
     if (L.tc) return launch_ffn_tc(fa, ws + L.xp, L.mcap, L.pad, num_sms(), stream, stages);
     if (L.decode) return launch_ffn_decode(fa, num_sms(), stream, stages);
     return launch_ffn_rowwise(fa, desc->dtype, num_sms(), stream, stages);
   };
   if (L.tc) {
-    GatherArgs ga{x, perm, hdr, ws + L.xp, desc->d, L.mcap};
+    // (the rows of the shared experts are x itself: gemm_rows.cu reads them there)
+    GatherArgs ga{x, perm, hdr, ws + L.xp, desc->d, L.mcap, L.rows ? off + E : nullptr};
     e = launch_gather(ga, stream);
     if (e != cudaSuccess) return cuda_fail(e, "gather kernel launch");
-    if (lora) {  // U13, GEMM13, U2 (from h), GEMM2
+    if (lora && !L.rows) {  // U13, GEMM13, U2 (from h), GEMM2
       e = launch_lora_down_tc(fa, ws + L.xp, L.mcap, num_sms(), stream, 1);
       if (e == cudaSuccess) e = ffn(1);
       if (e == cudaSuccess) e = launch_lora_down_tc(fa, ws + L.xp, L.mcap, num_sms(), stream, 2);
@@ -515,11 +533,11 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
       if (e != cudaSuccess) return cuda_fail(e, "LoRA expert GEMM launch");
     }
   }
-  if (!(lora && L.tc)) {
+  if (!(lora && L.tc && !L.rows)) {
     e = ffn(lora ? 1 : 3);
     if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
   }
-  if (lora && !L.tc) {
+  if (lora && (!L.tc || L.rows)) {
     // u2[q] = A2 h_q for every permuted row, then the down projection with its adapter
     const LoraOffsets lo = lora_offsets(desc->d, desc->w, lrank);
     la.in = fa.h;
@@ -530,7 +548,8 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     la.K = desc->w;
     la.u = const_cast<float*>(fa.u2);
     la.ustride = lrank;
-    e = launch_lora_down(la, desc->dtype, lrank, L.mcap, stream);
+    e = L.rows ? launch_lora_down_tiles(la, lrank, L.mcap, num_sms(), stream)
+               : launch_lora_down(la, desc->dtype, lrank, L.mcap, stream);
     if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
     e = ffn(2);
     if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
@@ -938,6 +957,14 @@ mcft_status mcft_moe_forward_cached(const mcft_layer_desc* desc, const void* x, 
 
 namespace mcft {
 
+mcft_status forward_decode_layout(const mcft_layer_desc* desc, const void* x, int T,
+                                  const int32_t* idx, const float* gate, const void* const* experts,
+                                  const void* const* shared, void* y, void* workspace,
+                                  size_t ws_bytes, cudaStream_t stream) {
+  return forward_impl(desc, x, T, idx, gate, experts, shared, nullptr, y, workspace, ws_bytes, stream,
+                      true);
+}
+
 mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int T,
                                 const int32_t* idx, const float* gate, mcft_cache* c, int layer,
                                 const void* const* shared, void* y, void* workspace,
@@ -965,7 +992,7 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
       ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15u))
     return fail(MCFT_ERR_INVALID, "misaligned x, y or workspace");
   const WsLayout L = ws_layout(desc->d, E, K, desc->w, S, desc->dtype, T);
-  if (L.tc)
+  if (L.tc && tc_aligned(desc->d, desc->w))
     return fail(MCFT_ERR_UNSUPPORTED, "T = %d runs the tensor-core path; use mcft_fetch_experts + "
                 "mcft_moe_forward", T);
   if (ws_bytes < L.total)
@@ -1088,7 +1115,7 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
     fa.phase = phase;
     if (phase == 2) MCFT_CUDA(cudaStreamWaitEvent(compute_stream, c->ev_copy, 0));
     const int reserved = phase == 1 || queued > 0 ? fetch_blocks() : 0;
-    e = L.decode ? launch_ffn_decode(fa, num_sms(), compute_stream, 3, reserved)
+    e = desc->dtype == MCFT_BF16 ? launch_ffn_decode(fa, num_sms(), compute_stream, 3, reserved)
                  : launch_ffn_rowwise(fa, desc->dtype, num_sms(), compute_stream);
     if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
   }

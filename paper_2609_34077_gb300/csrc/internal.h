@@ -78,13 +78,19 @@ struct WsLayout {
   int lrank;      // LoRA rank (0: no adapters)
   bool tc;        // tensor-core path (bf16, large T)
   bool decode;    // bf16 decode path (T <= 64)
-  int pad;        // rows per segment are padded to a multiple of this (TC path: 128, or 256
+  bool rows;      // tensor-core path with the weight rows on M (gemm_rows.cu): segments unpadded
+  int split;      // bf16 halves that keep a LoRA middle vector on that path
+  int pad;        // rows per segment are padded to a multiple of this (TC path: 1, 128, or 256
                   // for CTA-pair tiles)
   int mcap;       // capacity in permuted rows
   int ks;         // partial planes of o (contraction split of the decode GEMM2)
   size_t hdr, cnt, off, pos, perm, done, pscr, xp, h, o, u13, u2, total;
 };
-WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0);
+// no_tc: the layout of the decode kernels whatever T is.
+WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0,
+                   bool no_tc = false);
+// Layer sizes that fill the 128 x 256 tiles of gemm_tc.cu.
+inline bool tc_aligned(int d, int w) { return d % 256 == 0 && w % 128 == 0; }
 
 // LoRA adapter block of one expert (layer dtype, row-major), element offsets for rank r:
 // [A1 (r x d) | B1 (w x r) | A3 (r x d) | B3 (w x r) | A2 (r x w) | B2 (d x r)].
@@ -117,7 +123,11 @@ struct LoraDownArgs {
   int r, K;              // rank, contraction length
   float* u;              // output [mcap, ustride]
   int ustride;
+  float scale;           // tiles: U is scaled by it (lora_down leaves the scale to the epilogues)
+  int split;             // tiles: 1 = bf16 U, 2 = bf16 high and low halves
 };
+// The same on the tensor cores for large bf16 batches (U in bf16, see lora.cu), 16 rows per CTA.
+cudaError_t launch_lora_down_tiles(const LoraDownArgs& a, int outs, int mcap, int num_sms, cudaStream_t s);
 cudaError_t launch_lora_down(const LoraDownArgs& a, int dtype, int outs, int mcap, cudaStream_t s);
 
 struct PermuteArgs {
@@ -143,6 +153,7 @@ struct GatherArgs {
   const WsHeader* hdr;
   void* xp;       // [mcap, d] bf16
   int d, mcap;
+  const int* nrows;  // rows to gather (NULL: all, hdr->mrows)
 };
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s);
 
@@ -261,6 +272,10 @@ int decode_ksplit(int T);  // contraction split of the decode GEMM2 for T tokens
 cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, int num_sms,
                           cudaStream_t s, int stages = 3);
 bool tc_pair_tiles(int T, int K, int E, int lrank);
+// The expert GEMMs with the weight rows on M (gemm_rows.cu): any d and w, unpadded segments.
+// split: bf16 halves of the LoRA middle vectors (u13 / u2 as launch_lora_down_tiles wrote them).
+cudaError_t launch_ffn_rows(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s,
+                            int stages, int split);
 // Down projections of the adapters for the tcgen05 path, on the tensor cores, bf16 out scaled by
 // s: stage 1: u13[q] = s [A1 xp[q] | A3 xp[q]] (N = 2r); stage 2: u2[q] = s A2 h[q] (N = 16),
 // for the rows of every segment with an adapter. The expert GEMMs add the up projections.
@@ -417,6 +432,12 @@ cudaError_t launch_mask_grad(const MaskGradArgs& a, cudaStream_t s);
 
 unsigned* device_error_word();  // device address of the current device's error word
 mcft_status set_error_message(mcft_status st, const char* msg);  // mcft_last_error() text
+
+// mcft_moe_forward on the decode kernels and their workspace layout whatever T is (any d and w).
+mcft_status forward_decode_layout(const mcft_layer_desc* desc, const void* x, int T,
+                                  const int32_t* idx, const float* gate, const void* const* experts,
+                                  const void* const* shared, void* y, void* workspace,
+                                  size_t ws_bytes, cudaStream_t stream);
 
 // The device-driven cached forward (mcft_moe_forward_cached); permuted = the workspace already
 // holds this call's permutation (written by the fused prologue), so it is not recomputed.

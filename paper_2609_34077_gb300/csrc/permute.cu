@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads) permute_scatter_kernel(const __grid_
 __global__ void __launch_bounds__(256) gather_kernel(const __grid_constant__ GatherArgs a) {
   pdl_wait();
   if (a.hdr->abort) return;
-  const int mrows = a.hdr->mrows;
+  const int mrows = a.nrows ? *a.nrows : a.hdr->mrows;
   const int nch = a.d / 8;  // 16-byte chunks per row
   for (int r = blockIdx.x; r < mrows; r += gridDim.x) {
     const int t = a.perm[r];
