@@ -475,6 +475,7 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
   fa.o_plane = size_t(L.mcap) * desc->d;
   fa.ksplit = L.ks;
   fa.T = T;
+  fa.K = K;
   fa.d = desc->d;
   fa.w = desc->w;
   fa.nseg = E + S;
@@ -1036,6 +1037,7 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
     fa.o_plane = size_t(L.mcap) * desc->d;
     fa.ksplit = L.ks;
     fa.T = T;
+    fa.K = K;
     fa.d = desc->d;
     fa.w = desc->w;
     fa.nseg = E + S;
@@ -1101,6 +1103,7 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
   fa.o_plane = size_t(L.mcap) * desc->d;
   fa.ksplit = L.ks;
   fa.T = T;
+  fa.K = K;
   fa.d = desc->d;
   fa.w = desc->w;
   fa.nseg = E + S;

@@ -1,4 +1,5 @@
-// Row-streaming expert FFN for fp32 layers (CUDA-core fp32 arithmetic), plus the combine.
+// Row-streaming expert FFN for fp32 layers (CUDA-core fp32 arithmetic) with few rows per expert, plus
+// the combine.
 //
 // F(x) = W2 (silu(W1 x) * (W3 x)) per expert segment (Section 3.1; SwiGLU experts). Each weight
 // row is read once per call from HBM with 16-byte loads and dotted with every token of its segment
@@ -362,6 +363,12 @@ cudaError_t launch_combine_typed(const CombineArgs& a, cudaStream_t s) {
 
 cudaError_t launch_ffn_rowwise(const FfnArgs& a, int dtype, int num_sms, cudaStream_t s, int stages) {
   if (dtype != MCFT_F32) return cudaErrorInvalidValue;  // bf16 layers use the decode or TC path
+  // Rows an expert averages from which the 64-token tiles (ffn_tile.cu) win. Whole passes, row-wise
+  // against tiles: d 512, w 1024, 32 experts: 100 / 171 us at 4 rows, 142 / 177 at 8, 427 / 211 at 32;
+  // d 256, w 512: 64 experts 83 / 96 at 4, 117 / 100 at 8, 8 experts 348 / 60 at 128 (512 tokens).
+  // A function of the layer and the batch only, so every phase and path of a call takes the same.
+  constexpr int kTileMinRows = 12;
+  if (size_t(a.T) * a.K >= size_t(kTileMinRows) * a.E) return launch_ffn_tile(a, num_sms, s, stages);
   return launch_rowwise_typed<float>(a, num_sms, s, stages);
 }
 

@@ -166,7 +166,7 @@ struct FfnArgs {
   void* h;                       // [mcap, w] fp32 (rowwise) or bf16 (tensor cores, decode)
   float* o;                      // [ksplit][mcap, d] fp32
   size_t o_plane;                // elements between partial planes of o
-  int T, d, w, nseg, E, ksplit;
+  int T, K, d, w, nseg, E, ksplit;
   unsigned* err;
   // Expert addresses written on the device by a cache step (NULL: use wblk), that step's hit
   // mask, and which segments this launch computes: 0 all, 1 hit experts and shared experts,
@@ -262,6 +262,9 @@ __device__ __forceinline__ bool seg_in_phase(const FfnArgs& a, int s, unsigned l
 // stages: bit 0 = GEMM13 (+ SwiGLU), bit 1 = GEMM2
 cudaError_t launch_ffn_rowwise(const FfnArgs& a, int dtype, int num_sms, cudaStream_t s,
                                int stages = 3);  // fp32
+// The same in 64-token tiles (ffn_tile.cu): launch_ffn_rowwise passes it the calls whose routed
+// experts average enough rows.
+cudaError_t launch_ffn_tile(const FfnArgs& a, int num_sms, cudaStream_t s, int stages);
 // reserved: CTA slots left free for another kernel that may run at the same time (the expert
 // fetch, which otherwise could not start until the FFN's CTAs exit).
 cudaError_t launch_ffn_decode(const FfnArgs& a, int num_sms, cudaStream_t s, int stages = 3,
