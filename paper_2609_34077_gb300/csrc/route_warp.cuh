@@ -11,14 +11,10 @@
 
 namespace mcft {
 
-// Warp arg-max over (value, index) with ties to the lower index; ineligible = -inf and index E.
-__device__ __forceinline__ void warp_argmax(float& v, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    float v2 = __shfl_xor_sync(0xffffffffu, v, o);
-    int i2 = __shfl_xor_sync(0xffffffffu, i, o);
-    if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
-  }
+// A float as an integer of the same order (equal floats, 0 and -0 among them, give equal integers).
+__device__ __forceinline__ int ordered_int(float v) {
+  const int b = __float_as_int(v + 0.f);
+  return b ^ ((b >> 31) & 0x7fffffff);
 }
 
 // Called by one whole warp: zs = the token's E router logits (shared memory), t = its row in
@@ -46,25 +42,23 @@ __device__ inline void rank_and_gate_warp(const RouteArgs& a, const float* zs, i
       }
     }
   }
-  int sel_k[2] = {-1, -1};  // rank at which this lane's expert was selected
+  // Best first: a warp maximum of the scores' ordered integers (redux.sync), then the lowest expert
+  // index that holds it; INT_MIN, below every score, marks what is not eligible or already taken.
+  constexpr int kNone = -2147483647 - 1;
+  int key[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) key[j] = elig[j] ? ordered_int(s[j]) : kNone;
   float zsel = 0.f;
   int isel = 0;
   for (int k = 0; k < a.K; ++k) {
-    float v = -INFINITY;
-    int i = 1 << 30;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int e = lane + 32 * j;
-      if (elig[j] && sel_k[j] < 0 && (s[j] > v || (s[j] == v && e < i) || i == (1 << 30))) {
-        v = s[j];
-        i = e;
-      }
-    }
-    warp_argmax(v, i);
+    const int best = __reduce_max_sync(0xffffffffu, max(key[0], key[1]));
+    const unsigned lo = __ballot_sync(0xffffffffu, key[0] == best);
+    const unsigned hi = __ballot_sync(0xffffffffu, key[1] == best);
+    int i = lo ? __ffs(lo) - 1 : 31 + __ffs(hi);
 #pragma unroll
     for (int j = 0; j < 2; ++j)
-      if (lane + 32 * j == i) sel_k[j] = k;
-    if (i >= E) {  // fewer eligible experts than K: only reachable through NaN inputs
+      if (lane + 32 * j == i) key[j] = kNone;
+    if (best == kNone) {  // fewer eligible experts than K: only reachable through NaN inputs
       set_error(a.err, kErrInvalid);
       i = 0;
     }
