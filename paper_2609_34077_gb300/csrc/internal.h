@@ -55,7 +55,7 @@ struct RouteArgs {
 };
 cudaError_t launch_route(const RouteArgs& a, int dtype, cudaStream_t s);
 int num_sms();  // SMs of the current device (looked up once per device)
-// bf16 calls of more tokens than this route in 16-token tensor-core tiles (route.cu).
+// bf16 calls of more tokens than this route in tensor-core tiles (route.cu).
 constexpr int kRouteTileMinT = 64;
 
 // Header at the start of the forward workspace.

@@ -1,5 +1,6 @@
 // Router GEMV + mask / prior + Top-K + gate softmax: one CTA per token at decode sizes, tiles of
-// 16 tokens on the tensor cores at prefill sizes (route_tile_kernel, bf16).
+// 16 tokens (route_tile_kernel) or of 64 and 128 on clusters (route_tile_cluster_kernel) on the tensor
+// cores at prefill sizes (bf16).
 //
 // z = W x (Section 3.1); the score is z (plain Top-K, Eq. topk), z restricted to m_e = 1 (hard
 // mask, Eq. stage1) or z_e + log pi_e (soft prior, Eq. inference: log(p_e pi_e) = z_e + log pi_e
@@ -151,7 +152,7 @@ __global__ void __cluster_dims__(kRouteCluster, 1, 1) __launch_bounds__(kWarps *
   rank_and_gate_warp(a, zs, t);
 }
 
-// Prefill-sized bf16 calls (T > kRouteTileMinT): the router is a skinny GEMM z[T, E] = x W^T,
+// Prefill-sized bf16 calls (T > kRouteTileMinT) of few experts or short rows: the router is a skinny GEMM z[T, E] = x W^T,
 // bound by reading x once. A CTA of 8 warps takes up to 16 tokens; the logits come from mma.sync
 // m16n8k16 (bf16 products, exact in fp32, fp32 accumulation). The tokens are spread evenly over
 // two CTAs per SM (at most 16 per CTA, the MMA's rows; rows past a CTA's tokens read as zero), so
@@ -240,12 +241,201 @@ __global__ void __launch_bounds__(kTileWarps * 32, 2)
     if (t0 + t < t1) rank_and_gate_warp(a, zs[t], t0 + t);
 }
 
+// Prefill-sized bf16 calls of many experts and long rows: the same skinny GEMM z[T, E] = x W^T with
+// the contraction split over a cluster of 8 CTAs and 64 or 128 tokens per cluster. Each CTA copies its
+// slice of the token rows and of the router to shared memory (cp.async, 128 elements per stage, all of a
+// slice of up to 256 elements on its way at once), multiplies with mma.sync m16n8k16 (bf16 products,
+// exact in fp32, fp32 accumulation; with 64 tokens two warps share 16 tokens and take the k-steps in
+// turn), and leaves its partial logits in shared memory. After a cluster barrier every CTA ranks its
+// eighth of the tokens, one per warp: it adds the partial logits in a fixed order over distributed shared
+// memory. Rows past the last token or expert are zero-filled. The fp32 order differs from
+// route_kernel's by rounding only (about 1e-7 relative), far inside the near-tie band of the routing
+// contract.
+// Why: a router call is a chain of memory round trips. route_tile_kernel walks the contraction of its
+// tokens in passes of 34 loads per lane, four round trips at d = 2048 and E = 64, and reads the router
+// once per 16 tokens at most (75 MB from L2 at T = 4096, 51 MB at T = 200). In a replayed graph (GB300, d =
+// 2048, E = 64, K = 6), 16-token tiles against clusters: T = 200 11.7 / 7.1 us, 1000 12.1 / 8.9, 4096
+// 18.6 / 14.2, 16384 65.9 / 46.7; d = 4096, T = 4096 28.2 / 18.4. The floor at T = 4096 is 2.5 us of x from
+// HBM; what is left is the copy's, two cluster barriers' and the ranking's latency. Few experts or short
+// rows have one round trip to begin with: E = 8, d = 4096, T = 4096 9.5 / 11.5, E = 16, d = 960 4.5 / 5.1,
+// E = 33, d = 320 5.8 / 6.3, so they keep the tiles above. 128 tokens per cluster halve the CTAs where 64
+// would fill the GPU more than once (T = 4096 19.9 / 14.2 us; at 1000 8.9 / 9.4, so the line is 2048).
+constexpr int kClusterMinD = 1024;
+constexpr int kClusterWideT = 2048;
+constexpr int kTileCluster = 8;
+constexpr int kTileK = 128;       // contraction elements per stage
+constexpr int kTileMaxStages = 6;
+constexpr int kTileRingBytes = 98304;  // two CTAs per SM
+__host__ __device__ constexpr int route_tile_stage(int tt, int ntw) { return (tt + ntw * 8) * kTileK * 2; }
+
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t* r) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+// 16-byte copy to shared memory; zeros when `ok` is false (the address must still be readable).
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0)
+               : "memory");
+}
+
+// At most n commit groups pending (n <= 4, known at run time).
+__device__ __forceinline__ void cp_async_wait(int n) {
+  switch (n) {
+    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
+  }
+}
+
+template <int NTW, int TT>
+__global__ void __cluster_dims__(kTileCluster, 1, 1) __launch_bounds__(kTileWarps * 32, 2)
+    route_tile_cluster_kernel(const __grid_constant__ RouteArgs a, int depth) {
+  constexpr int NE = NTW * 8;         // expert columns, rows past E zero
+  constexpr int MT = TT / 16;         // 16-token MMA rows
+  constexpr int KH = kTileWarps / MT; // warps that share one of them, taking its k-steps in turn
+  constexpr int STAGE = route_tile_stage(TT, NTW);
+  // `depth` stages, over which the partial logits are laid once the products are done
+  extern __shared__ __align__(128) char smem[];
+  float(*part)[TT][NE + 1] = reinterpret_cast<float(*)[TT][NE + 1]>(smem);
+  __shared__ float zs[kTileWarps][kMaxE];
+  pdl_wait();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int crank = int(cluster.block_rank());
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int E = a.E, d = a.d;
+  const int t0 = int(blockIdx.x / kTileCluster) * TT;
+  // this CTA's contraction slice, in units of 64 elements (d is a multiple of 64)
+  const int units = d / 64, u0 = crank * units / kTileCluster, u1 = (crank + 1) * units / kTileCluster;
+  const int k0 = u0 * 64, len = (u1 - u0) * 64;
+  const int steps = (len + kTileK - 1) / kTileK;
+  const size_t row = size_t(d) * 2;
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+  // Copies: thread i takes 16-byte chunk c = i % 16 of rows i / 16, i / 16 + 16, ... of a stage. Stage
+  // rows are 256 bytes and chunk c of row r sits at chunk c ^ (r % 8), so the 8 rows of an ldmatrix hit
+  // different banks. One commit group per stage, empty past the end.
+  const int cr = tid >> 4, cc = tid & 15;
+  const char* xg = static_cast<const char*>(a.x) + size_t(k0 + cc * 8) * 2;
+  const char* wg = static_cast<const char*>(a.w_router) + size_t(k0 + cc * 8) * 2;
+  const uint32_t dst0 = base + cr * 256 + ((cc ^ (cr & 7)) << 4);  // (rows 16 apart share r % 8)
+  auto copy = [&](int st) {
+    if (st < steps) {
+      const uint32_t sb = dst0 + uint32_t(st % depth) * STAGE;
+      const bool in = st * kTileK + cc * 8 < len;
+      const size_t ko = in ? size_t(st) * kTileK * 2 : 0;
+#pragma unroll
+      for (int i = 0; i < TT / 16; ++i) {
+        const int t = t0 + cr + 16 * i;
+        const bool ok = in && t < a.T;
+        cp_async16z(sb + i * 4096, xg + size_t(ok ? t : 0) * row + (ok ? ko : 0), ok);
+      }
+#pragma unroll
+      for (int i = 0; i < (NE + 15) / 16; ++i) {
+        const int e = cr + 16 * i;
+        const bool ok = in && e < E;
+        if (e < NE) cp_async16z(sb + (TT + 16 * i) * 256, wg + size_t(ok ? e : 0) * row + (ok ? ko : 0), ok);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int st = 0; st < depth - 1; ++st) copy(st);
+  float acc[NTW][4];
+#pragma unroll
+  for (int j = 0; j < NTW; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.f;
+  const int mt = warp % MT, half = warp / MT;
+  const int arow = mt * 16 + (lane & 15);                                    // ldmatrix rows of A
+  const int brow = (lane & 7) + ((lane >> 4) << 3);  // and of B
+  for (int st = 0; st < steps; ++st) {
+    cp_async_wait(depth - 2);
+    __syncthreads();  // stage st has landed; everyone is done with stage st - 1
+    copy(st + depth - 1);
+    const uint32_t sb = base + uint32_t(st % depth) * STAGE;
+#pragma unroll
+    for (int s = 0; s < kTileK / 16 / KH; ++s) {
+      const int c = (KH * s + half) * 2;  // first 16-byte chunk of this warp's 16 elements
+      uint32_t af[4];
+      ldmatrix4(sb + arow * 256 + (((c + (lane >> 4)) ^ (arow & 7)) << 4), af);
+#pragma unroll
+      for (int j = 0; j < NTW; j += 2) {
+        uint32_t bf[4];
+        const int r = TT + j * 8 + brow;
+        ldmatrix4(sb + r * 256 + (((c + ((lane >> 3) & 1)) ^ (r & 7)) << 4), bf);
+        mma16816(acc[j], af[0], af[1], af[2], af[3], bf[0], bf[1]);
+        mma16816(acc[j + 1], af[0], af[1], af[2], af[3], bf[2], bf[3]);
+      }
+    }
+  }
+  __syncthreads();  // the stages are read
+  // C fragment of tile j: rows g and g + 8 (tokens), columns 2 c and 2 c + 1 (experts of the tile)
+  const int g = lane >> 2, c2 = (lane & 3) * 2;
+#pragma unroll
+  for (int j = 0; j < NTW; ++j) {
+    float* p = &part[half][mt * 16 + g][j * 8 + c2];
+    p[0] = acc[j][0];
+    p[1] = acc[j][1];
+    p[8 * (NE + 1)] = acc[j][2];
+    p[8 * (NE + 1) + 1] = acc[j][3];
+  }
+  cluster.sync();  // every CTA's partial logits are in its shared memory
+  // this CTA's tokens of the cluster's, one per warp and round
+#pragma unroll
+  for (int i = 0; i < TT / kTileCluster / kTileWarps; ++i) {
+    const int tl = crank * (TT / kTileCluster) + i * kTileWarps + warp;
+    if (t0 + tl >= a.T) break;
+    for (int e = lane; e < E; e += 32) {
+      float v[kTileCluster][KH];
+#pragma unroll
+      for (int r = 0; r < kTileCluster; ++r) {
+        const float* q = cluster.map_shared_rank(&part[0][tl][e], r);
+#pragma unroll
+        for (int h = 0; h < KH; ++h) v[r][h] = q[h * TT * (NE + 1)];
+      }
+      float z = 0.f;
+#pragma unroll
+      for (int r = 0; r < kTileCluster; ++r)
+#pragma unroll
+        for (int h = 0; h < KH; ++h) z += v[r][h];
+      zs[warp][e] = z;
+    }
+    __syncwarp();
+    rank_and_gate_warp(a, zs[warp], t0 + tl);
+    __syncwarp();
+  }
+  cluster.sync();  // no CTA leaves while another may still read its shared memory
+}
+
+template <int NTW, int TT>
+cudaError_t launch_route_tile_t(const RouteArgs& a, cudaStream_t s) {
+  constexpr int stage = route_tile_stage(TT, NTW), partial = 2 * 64 * (NTW * 8 + 1) * 4;
+  constexpr int most = kTileRingBytes / stage < kTileMaxStages ? kTileRingBytes / stage : kTileMaxStages;
+  static_assert(most >= 2, "the ring needs two stages");
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(route_tile_cluster_kernel<NTW, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           most * stage > partial ? most * stage : partial);
+  if (attr != cudaSuccess) return attr;
+  // a slice shorter than the ring takes one stage more than it has: all of it is copied at once
+  const int units = (a.d / 64 + kTileCluster - 1) / kTileCluster;
+  const int depth = max(2, min(most, (units * 64 + kTileK - 1) / kTileK + 1));
+  const int steps = (units * 64 + kTileK - 1) / kTileK;
+  const int smem = max(min(depth, steps) * stage, partial);
+  const dim3 grid((a.T + TT - 1) / TT * kTileCluster);
+  return launch_pdl(route_tile_cluster_kernel<NTW, TT>, grid, dim3(kTileWarps * 32), smem, s, a, depth);
+}
+template <int NTW>
+cudaError_t launch_route_tile_cluster(const RouteArgs& a, cudaStream_t s) {
+  return a.T <= kClusterWideT ? launch_route_tile_t<NTW, 64>(a, s) : launch_route_tile_t<NTW, 128>(a, s);
+}
+
 cudaError_t launch_route_tile(const RouteArgs& a, int num_sms, cudaStream_t s) {
   // tokens per CTA: the T tokens spread evenly over two CTAs per SM (at most 16, the MMA's rows)
   const int slots = 2 * num_sms;
   const int tpc = min(kTileTokens, max(1, (a.T + slots - 1) / slots));
   const dim3 grid((a.T + tpc - 1) / tpc), block(kTileWarps * 32);
   const int nt = (a.E + 7) / 8;
+  if (nt > 2 && a.d >= kClusterMinD)
+    return nt <= 4 ? launch_route_tile_cluster<4>(a, s) : launch_route_tile_cluster<8>(a, s);
   // chunks per pass: about 24 16-byte loads in flight per lane
   if (nt == 1) return launch_pdl(route_tile_kernel<1, 8>, grid, block, 0, s, a, tpc);
   if (nt == 2) return launch_pdl(route_tile_kernel<2, 6>, grid, block, 0, s, a, tpc);
@@ -259,7 +449,7 @@ cudaError_t launch_typed(const RouteArgs& a, cudaStream_t s) {
   const int per_lane = (nchunk / route_parts(a.E, nchunk) + 31) / 32;  // chunks per lane and task
   dim3 grid(a.T), block(kWarps * 32);
   prof_begin(kProfRoute, s);
-  if (sizeof(TX) == 2 && a.T > kRouteTileMinT) {  // prefill-sized: tensor-core tiles of 16 tokens
+  if (sizeof(TX) == 2 && a.T > kRouteTileMinT) {  // prefill-sized: tensor-core tiles
     const cudaError_t e = launch_route_tile(a, num_sms(), s);
     prof_end(kProfRoute, s);
     return e != cudaSuccess ? e : cudaGetLastError();
