@@ -171,7 +171,6 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   L.pos = o;  o = align256(o + sizeof(int) * size_t(T) * K);
   L.perm = o; o = align256(o + sizeof(int) * size_t(L.mcap));
   L.done = o; o = align256(o + sizeof(int) * (nseg + kClaimSlots));
-  L.pscr = o; o = align256(o + (T * K > kPermSingleMax ? sizeof(int) * kPermScrInts : 0));
   L.xp = o;   o = align256(o + (L.tc ? size_t(L.mcap) * d * 2 : 0));
   L.h = o;    o = align256(o + size_t(L.mcap) * w * (dtype == MCFT_BF16 ? 2 : 4));
   L.o = o;    o = align256(o + size_t(L.ks) * L.mcap * d * 4);
@@ -458,9 +457,15 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
 
   int* done = reinterpret_cast<int*>(ws + L.done);
   PermuteArgs pa{idx, T, K, E, S, L.pad, L.mcap, hdr, cnt, off, pos, perm, err, done,
-                 T * K > kPermSingleMax ? reinterpret_cast<int*>(ws + L.pscr) : nullptr};
+                 L.tc ? 1 : 0};
   cudaError_t e = launch_permute(pa, stream);
   if (e != cudaSuccess) return cuda_fail(e, "permute kernel launch");
+
+  if (L.tc) {
+    SpreadArgs sa{x, pos, perm, off, cnt, hdr, ws + L.xp, T, desc->d, K, E, S, L.pad};
+    e = launch_spread(sa, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "spread kernel launch");
+  }
 
   FfnArgs fa{};
   fa.x = x;
@@ -522,10 +527,6 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     return launch_ffn_rowwise(fa, desc->dtype, num_sms(), stream, stages);
   };
   if (L.tc) {
-    // (the rows of the shared experts are x itself: gemm_rows.cu reads them there)
-    GatherArgs ga{x, perm, hdr, ws + L.xp, desc->d, L.mcap, L.rows ? off + E : nullptr};
-    e = launch_gather(ga, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "gather kernel launch");
     if (lora && !L.rows) {  // U13, GEMM13, U2 (from h), GEMM2
       e = launch_lora_down_tc(fa, ws + L.xp, L.mcap, num_sms(), stream, 1);
       if (e == cudaSuccess) e = ffn(1);

@@ -84,7 +84,7 @@ struct WsLayout {
                   // for CTA-pair tiles)
   int mcap;       // capacity in permuted rows
   int ks;         // partial planes of o (contraction split of the decode GEMM2)
-  size_t hdr, cnt, off, pos, perm, done, pscr, xp, h, o, u13, u2, total;
+  size_t hdr, cnt, off, pos, perm, done, xp, h, o, u13, u2, total;
 };
 // no_tc: the layout of the decode kernels whatever T is.
 WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0,
@@ -140,22 +140,23 @@ struct PermuteArgs {
   int* perm;   // [mcap] token of each permuted row, -1 for padding
   unsigned* err;
   int* done;   // [E+S + kClaimSlots] progress and claim counters of the fused decode FFN, zeroed here
-  int* scr;    // NULL, or kPermScrInts of scratch: large batches then permute in chunks
+  int spread;  // T > kPermDecodeT: launch_spread follows and writes the routed rows of perm
 };
-constexpr int kPermChunks = 256;      // most chunks of the large-batch permutation
-constexpr int kPermSingleMax = 4096;  // up to this many assignments one CTA permutes (faster)
-constexpr int kPermScrInts = kPermChunks * kMaxE + kPermChunks;
+constexpr int kPermDecodeT = 64;  // up to this many tokens one CTA permutes
 cudaError_t launch_permute(const PermuteArgs& a, cudaStream_t s);
 
-struct GatherArgs {
+struct SpreadArgs {
   const void* x;  // [T, d] bf16
-  const int* perm;
+  const int* pos;
+  int* perm;      // routed rows written here
+  const int* off;
+  const int* cnt;
   const WsHeader* hdr;
   void* xp;       // [mcap, d] bf16
-  int d, mcap;
-  const int* nrows;  // rows to gather (NULL: all, hdr->mrows)
+  int T, d, K, E, S, pad;
+  int groups;     // warps that share a token's copies (set by launch_spread)
 };
-cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s);
+cudaError_t launch_spread(const SpreadArgs& a, cudaStream_t s);
 
 struct FfnArgs {
   const void* x;                 // [T, d] (FFN13) activations
