@@ -109,6 +109,11 @@ __device__ __forceinline__ void mma16816(float* d, uint32_t a0, uint32_t a1, uin
 
 __device__ __forceinline__ float silu(float u) { return u / (1.0f + expf(-u)); }
 
+// silu for results that are rounded to bf16 at once (2^-9): the quotient within 2 units of the last
+// fp32 place and without the division's branch for extreme operands, around which the compiler does
+// not interleave the many independent values of an epilogue thread.
+__device__ __forceinline__ float silu_to_bf16(float u) { return __fdividef(u, 1.0f + expf(-u)); }
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));

@@ -29,8 +29,9 @@
 //   rows included), GEMM2 68 -> 61 us.
 // * Mixtral shape, 4096 tokens (2048 rows an expert), GEMM13 1254 -> 1206 us, GEMM2 650 -> 703 us: the
 //   power cap bounds both, and there gemm_tc.cu keeps the large segments (see ws_layout).
-// Eight epilogue warps rather than four: the SwiGLU of a tile takes about 28,000 cycles on four, more
-// than the MMAs of a 2048-long contraction (16,400).
+// Eight epilogue warps rather than four, and a quotient without branches (silu_to_bf16): the SwiGLU of a
+// tile took about 28,000 cycles on four warps, more than the MMAs of a 2048-long contraction (16,400).
+// d = 960, w = 704 (15 k-blocks), 16 experts: GEMM13 at T = 4096 99 -> 63 us by the quotient alone.
 //
 // Roles (both CTAs of a pair): warp 0 TMA producer (its 128 weight rows and its half of the tokens,
 // counted on the leader's full[s]); warp 1 allocates TMEM and, in the leader, issues the MMAs; warps
@@ -383,7 +384,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             const uint32_t mine = low ? v[2 * i] : v[2 * i + 1];
             const uint32_t got = __shfl_xor_sync(0xffffffffu, low ? v[2 * i + 1] : v[2 * i], 16);
             const float g = __uint_as_float(low ? mine : got), u = __uint_as_float(low ? got : mine);
-            dst[i * kStgRow] = f2bf(silu(g) * u);  // two staging rows (2 * kStgRow bytes) per i
+            dst[i * kStgRow] = f2bf(silu_to_bf16(g) * u);  // two staging rows (2 * kStgRow bytes) per i
           }
           epi_sync(grp);  // one per chunk: a buffer is written again two chunks later
           const int col = (t.mt * 2 + int(rank)) * 64;

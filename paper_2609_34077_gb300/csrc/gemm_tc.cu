@@ -219,8 +219,8 @@ __device__ __forceinline__ void store_tile(const TcParams& p, uint8_t* stg, uint
         uint32_t pk[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-          pk[i] = pack2bf(silu(__uint_as_float(g[2 * i])) * __uint_as_float(u[2 * i]),
-                          silu(__uint_as_float(g[2 * i + 1])) * __uint_as_float(u[2 * i + 1]));
+          pk[i] = pack2bf(silu_to_bf16(__uint_as_float(g[2 * i])) * __uint_as_float(u[2 * i]),
+                          silu_to_bf16(__uint_as_float(g[2 * i + 1])) * __uint_as_float(u[2 * i + 1]));
         uint4* sw = reinterpret_cast<uint4*>(stg + lane * kOutRowBytes + c * 2);
         sw[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         sw[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
