@@ -8,7 +8,9 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from array import array
 
+import numpy as np
 import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libmcft.so")
@@ -101,21 +103,26 @@ def _check(st):
         raise MCFTError(st, lib().mcft_last_error().decode())
 
 
+# torch.cuda.current_stream() builds a Stream object for every call (3 us on a Grace core); the raw
+# handle of the same stream takes a tenth of that.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream):
     if stream is None:
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, torch.cuda.Stream):
-        return C.c_void_p(stream.cuda_stream)
-    return C.c_void_p(int(stream))
+        return stream.cuda_stream
+    return int(stream)
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return C.c_void_p(t)
+    if t is None or isinstance(t, int):
+        return t
     assert t.is_contiguous(), "tensors passed to libmcft must be contiguous"
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def desc_of(shape) -> LayerDesc:
@@ -143,18 +150,24 @@ def mcft_route(desc: LayerDesc, x, w_router, mode, mask=None, prior=None, idx=No
         idx = torch.empty((T, desc.K), dtype=torch.int32, device=x.device)
     if gate is None:
         gate = torch.empty((T, desc.K), dtype=torch.float32, device=x.device)
-    m = None
-    if mask is not None:
+    m = _host_array(mask, np.uint8, desc.E)
+    if m is None and mask is not None:
         mb = bytes(int(v) for v in mask)
         m = C.create_string_buffer(mb, len(mb))
-    p = None
-    if prior is not None:
+    p = _host_array(prior, np.float32, desc.E)
+    if p is None and prior is not None:
         p = (C.c_float * desc.E)(*[float(v) for v in prior])
-    _check(lib().mcft_route(C.byref(desc), _ptr(x), T, _ptr(w_router), int(mode),
-                            C.cast(m, C.c_void_p) if m is not None else None,
-                            C.cast(p, C.c_void_p) if p is not None else None,
-                            _ptr(idx), _ptr(gate), _stream(stream)))
+    _check(lib().mcft_route(C.byref(desc), _ptr(x), T, _ptr(w_router), int(mode), m, p, _ptr(idx),
+                            _ptr(gate), _stream(stream)))
     return idx, gate
+
+
+def _host_array(a, dtype, n):
+    """Address of a numpy array that already is n contiguous elements of dtype, else None (the library
+    reads mask and prior before it returns, so nothing is copied or kept)."""
+    if type(a) is np.ndarray and a.dtype == dtype and a.shape == (n,) and a.flags.c_contiguous:
+        return a.__array_interface__["data"][0]
+    return None
 
 
 def mcft_moe_workspace_size(desc: LayerDesc, T_max: int) -> int:
@@ -163,11 +176,24 @@ def mcft_moe_workspace_size(desc: LayerDesc, T_max: int) -> int:
     return n.value
 
 
+_data_ptr = torch.Tensor.data_ptr
+
+
 def _ptr_array(items, n):
-    arr = (C.c_void_p * max(n, 1))()
-    for i in range(n):
-        it = items[i] if items is not None and i < len(items) else None
-        arr[i] = None if it is None else (it if isinstance(it, int) else it.data_ptr())
+    """The first n addresses (of tensors, addresses or None; None past the end of items), as an array
+    whose memory a call reads at .buffer_info()[0]."""
+    if items is None:
+        items = ()
+    elif not isinstance(items, (list, tuple)):
+        items = [items[i] for i in range(min(n, len(items)))]
+    items = items[:n]
+    try:
+        arr = array("Q", map(_data_ptr, items))  # all tensors
+    except TypeError:
+        arr = array("Q", [0 if it is None else it if isinstance(it, int) else it.data_ptr()
+                          for it in items])
+    if len(arr) < max(n, 1):
+        arr.extend([0] * (max(n, 1) - len(arr)))
     return arr
 
 
@@ -183,7 +209,7 @@ def mcft_moe_forward(desc: LayerDesc, x, idx, gate, experts, shared=(), y=None, 
     ex = _ptr_array(experts, desc.E)
     sh = _ptr_array(shared, desc.n_shared)
     _check(lib().mcft_moe_forward(C.byref(desc), _ptr(x), T, _ptr(idx), _ptr(gate),
-                                  C.cast(ex, C.c_void_p), C.cast(sh, C.c_void_p), _ptr(y),
+                                  ex.buffer_info()[0], sh.buffer_info()[0], _ptr(y),
                                   _ptr(workspace), workspace.numel(), _stream(stream)))
     return y
 
@@ -208,8 +234,8 @@ def mcft_moe_forward_lora(desc: LayerDesc, x, idx, gate, experts, shared=(), exp
     el = _ptr_array(expert_lora, desc.E)
     sl = _ptr_array(shared_lora, desc.n_shared)
     _check(lib().mcft_moe_forward_lora(C.byref(desc), _ptr(x), T, _ptr(idx), _ptr(gate),
-                                       C.cast(ex, C.c_void_p), C.cast(sh, C.c_void_p),
-                                       C.cast(el, C.c_void_p), C.cast(sl, C.c_void_p), int(rank),
+                                       ex.buffer_info()[0], sh.buffer_info()[0],
+                                       el.buffer_info()[0], sl.buffer_info()[0], int(rank),
                                        float(scale), _ptr(y), _ptr(workspace), workspace.numel(),
                                        _stream(stream)))
     return y
@@ -224,7 +250,7 @@ def mcft_moe_forward_noalloc(desc: LayerDesc, x, idx, gate, experts, shared=(), 
     ex = _ptr_array(experts, desc.E)
     sh = _ptr_array(shared, desc.n_shared)
     _check(lib().mcft_moe_forward_noalloc(C.byref(desc), _ptr(x), T, _ptr(idx), _ptr(gate),
-                                          C.cast(ex, C.c_void_p), C.cast(sh, C.c_void_p), _ptr(y),
+                                          ex.buffer_info()[0], sh.buffer_info()[0], _ptr(y),
                                           _stream(stream)))
     return y
 
@@ -251,7 +277,7 @@ def mcft_cache_create(L, E, B, expert_bytes=0, host_experts=None, max_assign=102
     arr = _ptr_array(host_experts, L * E) if host_experts is not None else None
     pol = POLICY.get(policy, policy)
     _check(lib().mcft_cache_create(L, E, B, expert_bytes,
-                                   C.cast(arr, C.c_void_p) if arr is not None else None,
+                                   None if arr is None else arr.buffer_info()[0],
                                    max_assign, int(pol), C.byref(h)))
     c = Cache(h.value, L, E, B)
     c._host_experts = host_experts  # keep the pinned blocks alive
@@ -273,7 +299,7 @@ def mcft_fetch_experts(cache: Cache, layer, compute_stream=None, copy_stream=Non
     """Returns the E device addresses (0 for experts not selected this step)."""
     out = (C.c_void_p * cache.E)()
     _check(lib().mcft_fetch_experts(C.c_void_p(cache.handle), layer, _stream(compute_stream),
-                                    _stream(copy_stream), C.cast(out, C.c_void_p)))
+                                    _stream(copy_stream), out))
     return [v or 0 for v in out]
 
 
@@ -310,7 +336,7 @@ def mcft_moe_forward_cached(desc: LayerDesc, x, idx, gate, cache: Cache, layer, 
         workspace = torch.empty(mcft_moe_workspace_size(desc, T), dtype=torch.uint8, device=x.device)
     sh = _ptr_array(shared, desc.n_shared)
     _check(lib().mcft_moe_forward_cached(C.byref(desc), _ptr(x), T, _ptr(idx), _ptr(gate),
-                                         C.c_void_p(cache.handle), layer, C.cast(sh, C.c_void_p),
+                                         C.c_void_p(cache.handle), layer, sh.buffer_info()[0],
                                          _ptr(y), _ptr(workspace), workspace.numel(),
                                          _stream(compute_stream), _stream(copy_stream)))
     return y
@@ -321,7 +347,7 @@ def mcft_cache_last_misses(cache: Cache, layer):
     ex = (C.c_int32 * cache.E)()
     sl = (C.c_int32 * cache.E)()
     _check(lib().mcft_cache_last_misses(C.c_void_p(cache.handle), layer, C.byref(n),
-                                        C.cast(ex, C.c_void_p), C.cast(sl, C.c_void_p)))
+                                        ex, sl))
     return [(ex[i], sl[i]) for i in range(n.value)]
 
 
@@ -380,15 +406,14 @@ def mcft_stack_create(desc: LayerDesc, routers, priors, gammas, shared, eps, cac
     """routers, gammas: L device tensors; priors: [L, E] array-like (fp32 > 0); shared: L lists of
     S device blocks (or None when S = 0)."""
     L = len(routers)
-    import numpy as _np
-    pri = _np.ascontiguousarray(_np.asarray(priors, _np.float32).reshape(-1))
+    pri = np.ascontiguousarray(np.asarray(priors, np.float32).reshape(-1))
     rp = _ptr_array(routers, L)
     gp = _ptr_array(gammas, L)
     flat = [b for row in shared for b in row] if shared else []
     sp = _ptr_array(flat, len(flat))
     h = C.c_void_p()
-    _check(lib().mcft_stack_create(C.byref(desc), L, C.cast(rp, C.c_void_p), pri.ctypes.data,
-                                   C.cast(gp, C.c_void_p), C.cast(sp, C.c_void_p) if flat else None,
+    _check(lib().mcft_stack_create(C.byref(desc), L, rp.buffer_info()[0], pri.ctypes.data,
+                                   gp.buffer_info()[0], sp.buffer_info()[0] if flat else None,
                                    C.c_float(eps), C.c_void_p(cache.handle), int(n_prefetch),
                                    int(T_max), C.byref(h)))
     # keep everything the stack points to alive with it
@@ -405,11 +430,10 @@ def mcft_stack_step(stack: Stack, x, compute_stream=None, copy_stream=None):
 
 def mcft_stack_routing(stack: Stack, layer, stream=None):
     """(idx [T, K] int32, gate [T, K] fp32, idx_pred [T, K] int32) numpy copies of the last step."""
-    import numpy as _np
     T, K = stack.last_T, stack.K
-    idx = _np.empty((T, K), _np.int32)
-    gate = _np.empty((T, K), _np.float32)
-    pred = _np.empty((T, K), _np.int32)
+    idx = np.empty((T, K), np.int32)
+    gate = np.empty((T, K), np.float32)
+    pred = np.empty((T, K), np.int32)
     _check(lib().mcft_stack_routing(C.c_void_p(stack.handle), layer, idx.ctypes.data,
                                     gate.ctypes.data, pred.ctypes.data, _stream(stream)))
     return idx, gate, pred
@@ -423,7 +447,7 @@ def mcft_stack_destroy(stack: Stack):
 
 def mcft_cache_tags(cache: Cache, layer, stream=None):
     t = (C.c_int32 * cache.B)()
-    _check(lib().mcft_cache_tags(C.c_void_p(cache.handle), layer, C.cast(t, C.c_void_p),
+    _check(lib().mcft_cache_tags(C.c_void_p(cache.handle), layer, t,
                                  _stream(stream)))
     return list(t)
 
@@ -432,14 +456,14 @@ def mcft_cache_export(cache: Cache, stream=None) -> bytes:
     n = C.c_size_t(0)
     _check(lib().mcft_cache_export(C.c_void_p(cache.handle), None, C.byref(n), _stream(stream)))
     buf = C.create_string_buffer(n.value)
-    _check(lib().mcft_cache_export(C.c_void_p(cache.handle), C.cast(buf, C.c_void_p), C.byref(n),
+    _check(lib().mcft_cache_export(C.c_void_p(cache.handle), buf, C.byref(n),
                                    _stream(stream)))
     return buf.raw[: n.value]
 
 
 def mcft_cache_import(cache: Cache, state: bytes, stream=None):
     buf = C.create_string_buffer(state, len(state))
-    _check(lib().mcft_cache_import(C.c_void_p(cache.handle), C.cast(buf, C.c_void_p), len(state),
+    _check(lib().mcft_cache_import(C.c_void_p(cache.handle), buf, len(state),
                                    _stream(stream)))
 
 
@@ -474,8 +498,8 @@ def mcft_profile_read():
     names = (C.c_char_p * n.value)()
     launches = (C.c_uint64 * n.value)()
     ms = (C.c_double * n.value)()
-    _check(lib().mcft_profile_read(n.value, C.cast(names, C.c_void_p), C.cast(launches, C.c_void_p),
-                                   C.cast(ms, C.c_void_p), C.byref(n)))
+    _check(lib().mcft_profile_read(n.value, names, launches,
+                                   ms, C.byref(n)))
     return {names[i].decode(): (launches[i], ms[i]) for i in range(n.value)}
 
 
