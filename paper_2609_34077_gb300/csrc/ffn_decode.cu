@@ -690,6 +690,25 @@ int rows_per_item(int rows, int contraction, int rows_per_warp, int min_chunks =
   return rb;
 }
 
+// GEMM13 items grow further, up to 32 chunks per warp, while the segments the batch can have still make
+// 3.5 rounds of items over the two CTAs per SM: an item's reduction, publication and pipeline start
+// cost the same whatever its length (about 2 us of the 11 us of an 8-chunk item, during which its
+// CTA loads nothing), and with fewer rounds the last one weighs more than that. Decode passes (GB300), 8
+// chunks / this rule: Mixtral shape T = 2 165 / 160 us (16 chunks), 16 428 / 408 (32), 64 545 / 502; DeepSeek-
+// V2-Lite shape T = 16 126 / 122, 50 192 / 180, 64 216 / 203 (16). Past the line: T = 5 of the latter (2.3
+// rounds) 84 / 85, T = 2 of the former at 32 chunks (2.9 rounds) 165 / 170. GEMM2 items keep the minimum:
+// DeepSeek's at 16 chunks 191 -> 231 us of T = 50. The batch and the layer alone decide, as for every item
+// shape, so an output does not depend on which launch computes it.
+constexpr int kMaxChunks = 32;
+int widen_item(int rb, const FfnArgs& a, int num_sms) {
+  const long segs = min(long(a.T) * a.K, long(a.E)) + (a.nseg - a.E);
+  const int nch = a.d / kChunk;
+  while (rb < kWarps && a.w % (kRows * rb * 2) == 0 && nch / (kWarps / (2 * rb)) <= kMaxChunks &&
+         2 * segs * (a.w / (kRows * rb * 2)) >= 7L * 2 * num_sms)
+    rb *= 2;
+  return rb;
+}
+
 template <int MAXNG>
 cudaError_t launch_decode_ng(const FfnArgs& a, int num_sms, cudaStream_t s, int stages,
                              int reserved) {
@@ -698,7 +717,8 @@ cudaError_t launch_decode_ng(const FfnArgs& a, int num_sms, cudaStream_t s, int 
   // one CTA per SM slot, less the slots left to another kernel
   const int g13 = max(num_sms, num_sms * nb13 - reserved);
   const int g2 = max(num_sms, num_sms * nb2 - reserved);
-  const int rb13 = rows_per_item(a.w, a.d, kRows, a.T <= 4 ? kMinChunksSmallBatch : kMinChunks);
+  const int rb13 = widen_item(
+      rows_per_item(a.w, a.d, kRows, a.T <= 4 ? kMinChunksSmallBatch : kMinChunks), a, num_sms);
   const int rb2 = rows_per_item(a.d, a.w / a.ksplit, kRows2);
   cudaError_t e = cudaSuccess;
   if (stages == 3 && a.done && a.lrank == 0) {
