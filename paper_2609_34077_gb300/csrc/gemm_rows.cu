@@ -35,8 +35,9 @@
 //
 // Roles (both CTAs of a pair): warp 0 TMA producer (its 128 weight rows and its half of the tokens,
 // counted on the leader's full[s]); warp 1 allocates TMEM and, in the leader, issues the MMAs; warps
-// 2-9 read the CTA's 128 accumulator rows. Six stages of 32 KB, two accumulators of 256 columns, so a
-// tile's epilogue runs under the next tile's MMAs.
+// 2-9 read the CTA's 128 accumulator rows. A ring of 192 KB,
+// six stages of 32 KB with 256-token tiles and up to ten with narrower ones; two accumulators of 256
+// columns, so a tile's epilogue runs under the next tile's MMAs.
 //
 // With LoRA adapters (Section 3.2, Stage 2) an adapted tile appends p.nx k-blocks of one MMA each,
 // D += B' U^T: for GEMM13 B' is B1 on the gate rows (zeros on the up rows) with U = s A1 x, then B3 on
@@ -58,9 +59,9 @@ constexpr int kThreads = 64 + kEpiGroups * 128;
 constexpr int BK = 64;
 constexpr int kTileTok = 256;                 // most tokens of a tile
 constexpr int kBoxes = 4;                     // token boxes of 16, 32, 64 and 128 rows
-constexpr int kStages = 6;
+constexpr int kMaxStages = 10;
 constexpr int kABytes = 128 * BK * 2;         // a CTA's weight rows of a stage
-constexpr int kStageBytes = kABytes + (kTileTok / 2) * BK * 2;
+constexpr int kRingBytes = 6 * (kABytes + (kTileTok / 2) * BK * 2);
 constexpr int kTmemCols = 2 * kTileTok;
 constexpr int kMaxExtra = 4;
 // instruction descriptor without N: D fp32, A and B bf16, both K-major, M = 256
@@ -91,14 +92,14 @@ struct RowsLoraParams : RowsParams {
 };
 
 struct Ctl {
-  uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], drain;
+  uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
   uint32_t tmem_base;
-  int abort, tiles;
+  int abort, tiles, stages, stage_bytes;
   int off[kMaxSeg + 1];
   int first[kMaxSeg + 1];  // by position (segments in reverse order): first tile
 };
 constexpr int kCtlBytes = (int(sizeof(Ctl)) + 15) / 16 * 16;
-constexpr int kSmem = kStages * kStageBytes + 1024 + kCtlBytes + 2 * kEpiGroups * kStgBytes;
+constexpr int kSmem = kRingBytes + 1024 + kCtlBytes + 2 * kEpiGroups * kStgBytes;
 static_assert(kSmem <= 227 * 1024, "shared memory");
 
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, int c0,
@@ -140,6 +141,11 @@ __device__ __forceinline__ int epi_all(int grp, int v) {
 }
 
 __device__ __forceinline__ int token_tiles(int rows) { return (rows + kTileTok - 1) / kTileTok; }
+// Tokens of a segment's tiles, all but the last one's: equal shares, rounded up to 32.
+__device__ __forceinline__ int tile_tokens(int rows) {
+  const int nt = max(token_tiles(rows), 1);
+  return ((rows + nt - 1) / nt + 31) & ~31;
+}
 
 struct TileAt {
   int seg, mt, row0, n;  // segment, weight tile, first permuted row, tokens
@@ -161,7 +167,7 @@ __device__ __forceinline__ TileAt tile_at(const Ctl* c, int nseg, int mtiles, in
   const int local = tile - c->first[lo];
   const int rows = c->off[t.seg + 1] - c->off[t.seg];
   const int nt = token_tiles(rows);
-  const int ts = ((rows + nt - 1) / nt + 31) & ~31;  // (nt - 1) * ts < rows, since ts <= 256
+  const int ts = tile_tokens(rows);  // (nt - 1) * ts < rows, since ts <= 256
   const int g = local / (group_x * mtiles);
   const int r = local - g * group_x * mtiles;
   const int gsz = min(group_x, nt - g * group_x);
@@ -181,14 +187,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;  // the same offsets in both CTAs
-  Ctl* ctl = reinterpret_cast<Ctl*>(smem_raw + (base - raw) + kStages * kStageBytes);
+  Ctl* ctl = reinterpret_cast<Ctl*>(smem_raw + (base - raw) + kRingBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   const int nseg = p.nseg;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(&ctl->full[s], 1);
       mbar_init(&ctl->empty[s], 1);
     }
@@ -218,7 +224,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       if (s <= nseg) ctl->off[s] = p.off[s];
     }
     __syncwarp();
-    int cnt[3], sum = 0;
+    int cnt[3], sum = 0, wide = 0;
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -227,7 +233,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       bad |= rows > 0 && !in_mask(p.wmask, s);  // a selected expert without weights
       cnt[j] = token_tiles(rows) * p.mtiles;
       sum += cnt[j];
+      wide = max(wide, tile_tokens(rows));
     }
+    wide = __reduce_max_sync(0xffffffffu, wide);
     int incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -250,6 +258,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       ctl->abort = stop ? 1 : 0;
       ctl->tiles = stop ? 0 : incl;
+      ctl->stage_bytes = kABytes + wide / 2 * BK * 2;
+      ctl->stages = min(kMaxStages, kRingBytes / ctl->stage_bytes);
     }
   }
   tc_fence_before();
@@ -260,6 +270,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const int tiles = ctl->tiles;
   const int cid = int(blockIdx.x >> 1), ncl = int(gridDim.x >> 1);  // pair, pairs
   volatile int* abort = &ctl->abort;
+  const int stages = ctl->stages, stage_bytes = ctl->stage_bytes;
   // k-blocks of a segment's tiles: the contraction, then the adapter's extra ones
   auto extra_of = [&](int seg) -> int {
     if constexpr (LORA) return in_mask(p.lmask, seg) ? p.nx : 0;
@@ -268,7 +279,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0 && cid < tiles) {
-      uint32_t it = 0;
+      int s = 0, issued = 0;
+      uint32_t ph = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
         const TileAt t = tile_at(ctl, nseg, p.mtiles, p.group_x, tile);
         const int half = t.cols() / 2;
@@ -277,10 +289,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const int urow = t.row0 + int(rank) * half;
         const int nkb = p.kblocks + extra_of(t.seg);
         const uint32_t bytes = 2u * uint32_t(kABytes + half * BK * 2);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = int(it % kStages);
-          if (!mbar_wait_cl(&ctl->empty[s], ((it / kStages) & 1u) ^ 1u, abort, p.err)) break;
-          const uint32_t sa = base + uint32_t(s) * kStageBytes, sb = sa + kABytes;
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait_cl(&ctl->empty[s], ph ^ 1u, abort, p.err)) break;
+          const uint32_t sa = base + uint32_t(s * stage_bytes), sb = sa + kABytes;
           const uint32_t fb = peer_addr(&ctl->full[s], 0);
           if (leader) mbar_expect_tx(&ctl->full[s], bytes);
           const CUtensorMap* mw = &p.w[t.seg];
@@ -307,19 +318,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
               tma_load_2d_pair(sb + uint32_t(r) * (BK * 2), mx + b, c0, row + r, fb);
               r += 16 << b;
             }
+          if (issued < stages) ++issued;
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
       }
       // Stages still in flight: the leader waits for their bytes (both CTAs'), the peer until the
       // leader's MMAs consumed them; after the first wait that runs out the rest are skipped.
-      const uint32_t n_tail = it < kStages ? it : kStages;
-      for (uint32_t j = it - n_tail; j < it; ++j) {
-        uint64_t* bar = leader ? &ctl->full[j % kStages] : &ctl->empty[j % kStages];
-        if (!mbar_wait_drain_cl(bar, (j / kStages) & 1u, p.err)) break;
+      // (oldest first: the stages before s in this round of the ring, those from s on in the last one)
+      for (int i = 0; i < issued; ++i) {
+        const int back = issued - i, j = s - back;
+        uint64_t* ring = leader ? ctl->full : ctl->empty;
+        if (!mbar_wait_drain_cl(&ring[j < 0 ? j + stages : j], j < 0 ? ph ^ 1u : ph, p.err)) break;
       }
     }
   } else if (warp == 1) {
     if (leader && lane == 0 && cid < tiles) {
-      uint32_t it = 0, lt = 0;
+      int s = 0;
+      uint32_t ph = 0, lt = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
         const TileAt t = tile_at(ctl, nseg, p.mtiles, p.group_x, tile);
         const uint32_t idesc = kIdesc | (uint32_t(t.cols() >> 3) << 17);
@@ -329,14 +347,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tc_fence_after();
         const uint32_t dt = tmem + b * kTileTok;
         bool ok = true;
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = int(it % kStages);
-          if (!mbar_wait_cl(&ctl->full[s], (it / kStages) & 1u, abort, p.err)) {
+        for (int kb = 0; kb < nkb; ++kb) {
+          if (!mbar_wait_cl(&ctl->full[s], ph, abort, p.err)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = base + uint32_t(s) * kStageBytes, sb = sa + kABytes;
+          const uint32_t sa = base + uint32_t(s * stage_bytes), sb = sa + kABytes;
           const uint64_t da = sw128_desc(sa), db = sw128_desc(sb);
           if (!LORA || kb < p.kblocks) {
 #pragma unroll
@@ -347,6 +364,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             tc_mma_pair(dt, da, db, idesc, 1u);
           }
           tc_commit_pair_both(&ctl->empty[s]);
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
         if (!ok) break;
         tc_commit_pair_both(&ctl->tfull[b]);
