@@ -512,13 +512,9 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     la.ustride = 2 * lrank;
     la.scale = lora->scale;
     la.split = L.split;
-    if (L.rows) {
-      e = launch_lora_down_tiles(la, 2 * lrank, L.mcap, num_sms(), stream);
-      if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
-    } else if (!L.tc) {  // the padded tiles project the gathered rows instead, after the gather
-      e = launch_lora_down(la, desc->dtype, 2 * lrank, L.mcap, stream);
-      if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
-    }
+    e = L.tc ? launch_lora_down_tiles(la, 2 * lrank, L.mcap, num_sms(), stream)
+             : launch_lora_down(la, desc->dtype, 2 * lrank, L.mcap, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
   }
   auto ffn = [&](int stages) -> cudaError_t {
     if (L.rows) return launch_ffn_rows(fa, ws + L.xp, L.mcap, num_sms(), stream, stages, L.split);
@@ -526,20 +522,9 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     if (L.decode) return launch_ffn_decode(fa, num_sms(), stream, stages);
     return launch_ffn_rowwise(fa, desc->dtype, num_sms(), stream, stages);
   };
-  if (L.tc) {
-    if (lora && !L.rows) {  // U13, GEMM13, U2 (from h), GEMM2
-      e = launch_lora_down_tc(fa, ws + L.xp, L.mcap, num_sms(), stream, 1);
-      if (e == cudaSuccess) e = ffn(1);
-      if (e == cudaSuccess) e = launch_lora_down_tc(fa, ws + L.xp, L.mcap, num_sms(), stream, 2);
-      if (e == cudaSuccess) e = ffn(2);
-      if (e != cudaSuccess) return cuda_fail(e, "LoRA expert GEMM launch");
-    }
-  }
-  if (!(lora && L.tc && !L.rows)) {
-    e = ffn(lora ? 1 : 3);
-    if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
-  }
-  if (lora && (!L.tc || L.rows)) {
+  e = ffn(lora ? 1 : 3);
+  if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
+  if (lora) {
     // u2[q] = A2 h_q for every permuted row, then the down projection with its adapter
     const LoraOffsets lo = lora_offsets(desc->d, desc->w, lrank);
     la.in = fa.h;
@@ -550,8 +535,8 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     la.K = desc->w;
     la.u = const_cast<float*>(fa.u2);
     la.ustride = lrank;
-    e = L.rows ? launch_lora_down_tiles(la, lrank, L.mcap, num_sms(), stream)
-               : launch_lora_down(la, desc->dtype, lrank, L.mcap, stream);
+    e = L.tc ? launch_lora_down_tiles(la, lrank, L.mcap, num_sms(), stream)
+             : launch_lora_down(la, desc->dtype, lrank, L.mcap, stream);
     if (e != cudaSuccess) return cuda_fail(e, "LoRA kernel launch");
     e = ffn(2);
     if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");

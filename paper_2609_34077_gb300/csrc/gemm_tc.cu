@@ -6,10 +6,9 @@
 //           h[m, n0:n0+128] = bf16(silu(acc_gate) * acc_up)             (fused epilogue)
 //   GEMM2:  o[m, n0:n0+256] = h[m] . W2[n0:n0+256]^T                       (fp32 out)
 // both D = A B^T with A and B K-major bf16, fp32 accumulators in tensor memory.
-// With LoRA adapters (Section 3.2, Stage 2) every projection is W v + s B (A v). The down
-// projections are skinny GEMMs on the same kernel (N = 16 or 32 columns, bf16 out, scaled by s):
-//   DOWN13: U13[m] = s [A1 xp[m] | A3 xp[m]]    DOWN2: U2[m] = s A2 h[m]
-// and the up projections ride on the expert GEMMs as one extra k-block per adapted tile,
+// With LoRA adapters (Section 3.2, Stage 2) every projection is W v + s B (A v). The down projections
+// U13[m] = s [A1 xp[m] | A3 xp[m]] and U2[m] = s A2 h[m] come from lora.cu in bf16, and the up
+// projections ride on the expert GEMMs as one extra k-block per adapted tile,
 // D += U B'^T, so the tensor cores add them to the accumulators and the epilogues are unchanged.
 //
 // One persistent CTA per SM, 6 warps (7 with adapters):
@@ -22,8 +21,6 @@
 //             shared memory and stored as whole 128-byte row segments; they release the
 //             accumulator so the next tile's MMAs overlap this tile's epilogue;
 //   warp 6  - with adapters only: writes each adapted tile's extra k-block (see LoraOps).
-// The down projections use the same roles with N = 16 or 32: 8 stages of 18-20 KB, 32 or 64 TMEM
-// columns, bf16 rows written directly.
 // Tiles are walked m-fastest inside groups of m-tiles so concurrently running CTAs share weight
 // tiles (and the activation group) in L2. Every wait is bounded: after 2 s the kernel records
 // MCFT_ERR_TIMEOUT, stops issuing, waits (bounded) for its copies and MMAs in flight, frees TMEM
@@ -40,12 +37,12 @@ namespace {
 
 constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 6;  // of the pair tiles
 constexpr int kThreads = 192;  // producer, MMA, 4 epilogue warps
 constexpr int kBuilderWarp = 6;  // with adapters: one more warp writes the extra k-blocks
 __host__ __device__ constexpr int threads_for(int lr) { return lr > 0 ? kThreads + 32 : kThreads; }
 
-enum { EPI_SWIGLU = 0, EPI_F32 = 1, EPI_DOWN = 2 };
+enum { EPI_SWIGLU = 0, EPI_F32 = 1 };
 
 struct TcParams {
   CUtensorMap tma_a;
@@ -58,13 +55,10 @@ struct TcParams {
   int nseg, kblocks, ntiles_n, ldo, b_half, group_m;
   // LoRA (Stage 2): adapter block per segment (NULL: none); lug: the U operand rows (bf16;
   // GEMM13 [rows, 2r] = s [A1 x | A3 x], GEMM2 [rows, r] = s A2 h); lb0 / lb1: element offsets
-  // of the up matrices (B1, B3 for GEMM13; B2 for GEMM2); lscale = s = alpha / r (DOWN scales
-  // its output by it). b3d: the DOWN B map is 3-D ([A1; A3] planes) rather than 2-D (A2).
+  // of the up matrices (B1, B3 for GEMM13; B2 for GEMM2).
   const char* lblk[kMaxSeg];
   const uint16_t* lug;
   size_t lb0, lb1;
-  float lscale;
-  int b3d;
 };
 
 struct SmemCtl {
@@ -77,30 +71,26 @@ struct SmemCtl {
   int off[kMaxSeg + 1];
 };
 
-// Geometry for an N-tile of NB columns: the expert GEMMs use NB = 256 (4 stages of 48 KB, two
-// 128 x 256 fp32 accumulators = all 512 TMEM columns); the adapter down projection NB = 2r
-// (8 stages of 18-20 KB, 32 or 64 TMEM columns).
-// Epilogue store staging of the expert GEMMs: each epilogue warp writes 32 rows x 128 bytes of its
+// Geometry: 4 stages of 48 KB, two 128 x 256 fp32 accumulators = all 512 TMEM columns.
+// Epilogue store staging: each epilogue warp writes 32 rows x 128 bytes of its
 // output into shared memory (rows padded to 144 bytes: conflict-free 16-byte writes and reads),
 // then stores them as whole 128-byte row segments, four rows per instruction.
 constexpr int kOutRowBytes = 144;
 constexpr int kOutWarpBytes = 32 * kOutRowBytes;
 constexpr int kCtlBytes = (int(sizeof(SmemCtl)) + 15) / 16 * 16;
 
-template <int NB>
 struct Tile {
+  static constexpr int NB = BN;
   static constexpr int B_BYTES = NB * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = NB >= 128 ? 4 : kMaxStages;
-  static constexpr int TMEM_COLS = 2 * NB < 32 ? 32 : 2 * NB;
+  static constexpr int STAGES = 4;
+  static constexpr int TMEM_COLS = 2 * NB;
   // Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A bf16 (bits 7-9 = 1), B bf16
   // (bits 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
   static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
                                     (uint32_t(NB >> 3) << 17) | (uint32_t(BM >> 4) << 24);
-  static constexpr int OUT_STAGE = NB >= 128 ? 4 * kOutWarpBytes : 0;
+  static constexpr int OUT_STAGE = 4 * kOutWarpBytes;
   static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + kCtlBytes + OUT_STAGE;
-  static_assert(NB % 16 == 0 && NB >= 16 && NB <= 256, "M = 128 needs N a multiple of 16");
-  static_assert((TMEM_COLS & (TMEM_COLS - 1)) == 0 && TMEM_COLS <= 512, "TMEM allocation");
   static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
@@ -118,15 +108,6 @@ __device__ __forceinline__ int seg_of_row(const SmemCtl* c, int row) {
   int s = 0;
   while (s + 1 < c->nseg && c->off[s + 1] <= row) ++s;
   return s;
-}
-
-// Whether an m-tile has work: always for the expert GEMMs; for the adapter down projection only
-// when its segment (expert) has an adapter.
-template <int EPI>
-__device__ __forceinline__ bool tile_live(const SmemCtl* c, const TcParams& p, int mt) {
-  if constexpr (EPI != EPI_DOWN) return true;
-  const int s = seg_of_row(c, mt * BM);
-  return ((p.wmask[s >> 5] >> (s & 31)) & 1u) != 0;
 }
 
 // The adapter operands of the extra k-block an adapted tile appends to its K loop (the up
@@ -261,13 +242,13 @@ __device__ __forceinline__ void store_tile(const TcParams& p, uint8_t* stg, uint
   }
 }
 
-template <int EPI, int LR, int NB>
+template <int EPI, int LR>
 __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
-  using C = Tile<NB>;
+  using C = Tile;
+  constexpr int NB = C::NB;
   constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, TMEM_COLS = C::TMEM_COLS;
   constexpr int LRA = LR > 0 ? LR : 8;
   using LOps = LoraOps<EPI, LRA>;
-  static_assert(LR == 0 || NB == BN, "adapters ride on the expert GEMMs");
   pdl_wait();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -280,7 +261,7 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
     const int nseg = p.nseg;
     ctl->nseg = nseg;
     for (int s = 0; s <= nseg; ++s) ctl->off[s] = p.off[s];
-    for (int s = 0; s < nseg && EPI != EPI_DOWN; ++s) {  // no adapter: no down projection
+    for (int s = 0; s < nseg; ++s) {
       if (ctl->off[s + 1] > ctl->off[s] && !((p.wmask[s >> 5] >> (s & 31)) & 1u)) {
         set_error(p.err, kErrInvalid);  // a selected expert without weights
         const_cast<WsHeader*>(p.hdr)->abort = 1;  // later kernels of the call skip their work
@@ -330,7 +311,6 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
       for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x) {
         int mt, nt;
         tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-        if (!tile_live<EPI>(ctl, p, mt)) continue;
         const int row0 = mt * BM;
         const int sg = seg_of_row(ctl, row0);
         const CUtensorMap* mb = &p.tma_b[sg];
@@ -342,15 +322,8 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
           const uint32_t sa = base + uint32_t(s) * STAGE_BYTES, sb = sa + A_BYTES;
           mbar_expect_tx(&ctl->full[s], STAGE_BYTES);
           tma_load_2d(sa, &p.tma_a, kb * BK, row0, &ctl->full[s]);
-          if constexpr (EPI == EPI_DOWN) {
-            if (p.b3d)  // [A1; A3]: one box of r rows x 2 planes
-              tma_load_3d(sb, mb, kb * BK, 0, 0, &ctl->full[s]);
-            else        // A2: a box of NB rows, those past r zero-filled
-              tma_load_2d(sb, mb, kb * BK, 0, &ctl->full[s]);
-          } else {
-            tma_load_2d(sb, mb, kb * BK, yb0, &ctl->full[s]);
-            tma_load_2d(sb + C::B_BYTES / 2, mb, kb * BK, yb1, &ctl->full[s]);
-          }
+          tma_load_2d(sb, mb, kb * BK, yb0, &ctl->full[s]);
+          tma_load_2d(sb + C::B_BYTES / 2, mb, kb * BK, yb1, &ctl->full[s]);
         }
         if constexpr (LR > 0) {
           if (p.lblk[sg] != nullptr && !*abort) {  // the extra k-block's stage, for the builder
@@ -401,11 +374,10 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
       uint32_t it = 0, lt = 0;
       for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x) {
         bool lor = false;
-        if constexpr (EPI == EPI_DOWN || LR > 0) {
+        if constexpr (LR > 0) {
           int mt, nt;
           tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-          if (!tile_live<EPI>(ctl, p, mt)) continue;
-          if constexpr (LR > 0) lor = p.lblk[seg_of_row(ctl, mt * BM)] != nullptr;
+            lor = p.lblk[seg_of_row(ctl, mt * BM)] != nullptr;
         }
         const uint32_t b = lt & 1u;
         if (!mbar_wait(&ctl->tempty[b], ((lt >> 1) & 1u) ^ 1u, abort, p.err)) break;
@@ -443,12 +415,10 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
     }
   } else if (warp >= 2 && warp < 6) {
     const int q = warp & 3;  // TMEM lane quarter this warp may access
-    const int row = q * 32 + lane;
     uint32_t lt = 0;
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       int mt, nt;
       tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-      if (!tile_live<EPI>(ctl, p, mt)) continue;
       const uint32_t b = lt & 1u;
       int ok = 1;
       if (lane == 0) ok = mbar_wait(&ctl->tfull[b], (lt >> 1) & 1u, abort, p.err) ? 1 : 0;
@@ -456,29 +426,10 @@ __global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __gri
       if (!ok) break;
       tc_fence_after();
       const uint32_t taddr = tmem + b * NB + (uint32_t(q * 32) << 16);
-      const size_t grow = size_t(mt) * BM + row;
       // this warp's staging rows; row r of the warp's quarter goes to global row grow0 + r
       uint8_t* stg = reinterpret_cast<uint8_t*>(ctl) + kCtlBytes + q * kOutWarpBytes;
       const size_t grow0 = size_t(mt) * BM + q * 32;
-      if constexpr (EPI == EPI_DOWN) {  // U = s (A v) in bf16, the first ldo columns
-        uint16_t* out = reinterpret_cast<uint16_t*>(p.out) + grow * p.ldo;
-#pragma unroll
-        for (int c = 0; c < NB; c += 16) {
-          uint32_t v[16];
-          tmem_ld16(taddr + c, v);
-          tmem_ld_wait();
-          uint32_t pk[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            pk[i] = pack2bf(p.lscale * __uint_as_float(v[2 * i]),
-                            p.lscale * __uint_as_float(v[2 * i + 1]));
-          uint4* dst = reinterpret_cast<uint4*>(out + c);
-          dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-          if (c + 16 <= p.ldo) dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        }
-      } else {
-        store_tile<EPI, NB>(p, stg, taddr, grow0, nt, lane);
-      }
+      store_tile<EPI, NB>(p, stg, taddr, grow0, nt, lane);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->tempty[b]);
@@ -687,36 +638,6 @@ bool encode_2d(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The [A1; A3] rows of one adapter block as a 3-D map {d, r, 2}: plane 0 = A1 (element offset
-// 0), plane 1 = A3 (plane stride a3 elements); box 64 columns x r rows x 2 planes, so one load
-// fills the 2r rows of a down-projection B tile (A1 rows first), 128-byte swizzle.
-bool encode_adapter_a13(CUtensorMap* m, const void* blk, uint64_t d, uint32_t r, uint64_t a3) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn || (reinterpret_cast<uintptr_t>(blk) & 15u) || ((d * 2) & 15u) || ((a3 * 2) & 15u))
-    return false;
-  const cuuint64_t dims[3] = {d, r, 2};
-  const cuuint64_t strides[2] = {d * 2, a3 * 2};
-  const cuuint32_t box[3] = {BK, r, 2};
-  const cuuint32_t es[3] = {1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(blk), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// A2 of one adapter block, [r, w] row-major, as a 2-D map with a box of 64 columns x 16 rows:
-// for r = 8 the rows past r are outside the tensor and arrive as zeros (an N = 16 B tile).
-bool encode_adapter_a2(CUtensorMap* m, const void* a2, uint64_t w, uint32_t r) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn || (reinterpret_cast<uintptr_t>(a2) & 15u) || ((w * 2) & 15u) || r > 16) return false;
-  const cuuint64_t dims[2] = {w, r};
-  const cuuint64_t strides[1] = {w * 2};
-  const cuuint32_t box[2] = {BK, 16};
-  const cuuint32_t es[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a2), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 constexpr size_t kSmallSegGroupMB = 2;  // group budget when routed experts have few m-tiles
 // With CTA-pair tiles selected, layers whose routed experts average at least this many rows run
 // on pairs (segments padded to 256 rows); with fewer the extra padding would dominate.
@@ -728,14 +649,14 @@ int group_for(size_t a_tile_bytes, size_t budget_mb) {
   return g < 1 ? 1 : int(g > 4096 ? 4096 : g);
 }
 
-template <int EPI, int LR, int NB>
+template <int EPI, int LR>
 cudaError_t launch_one(const TcParams& p, int grid, cudaStream_t s) {
   static cudaError_t attr = cudaFuncSetAttribute(
-      gemm_tc_kernel<EPI, LR, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile<NB>::SMEM);
+      gemm_tc_kernel<EPI, LR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile::SMEM);
   if (attr != cudaSuccess) return attr;
-  const int kid = EPI == EPI_SWIGLU ? kProfGemm13 : EPI == EPI_F32 ? kProfGemm2 : kProfLora;
+  const int kid = EPI == EPI_SWIGLU ? kProfGemm13 : kProfGemm2;
   prof_begin(kid, s);
-  gemm_tc_kernel<EPI, LR, NB><<<grid, threads_for(LR), Tile<NB>::SMEM, s>>>(p);
+  gemm_tc_kernel<EPI, LR><<<grid, threads_for(LR), Tile::SMEM, s>>>(p);
   prof_end(kid, s);
   return cudaGetLastError();
 }
@@ -770,9 +691,9 @@ cudaError_t launch_pair(const TcParams& p, int num_sms, cudaStream_t s) {
 template <int EPI>
 cudaError_t launch_rank(const TcParams& p, int rank, int num_sms, cudaStream_t s) {
   switch (rank) {
-    case 0: return launch_one<EPI, 0, BN>(p, num_sms, s);
-    case 8: return launch_one<EPI, 8, BN>(p, num_sms, s);
-    case 16: return launch_one<EPI, 16, BN>(p, num_sms, s);
+    case 0: return launch_one<EPI, 0>(p, num_sms, s);
+    case 8: return launch_one<EPI, 8>(p, num_sms, s);
+    case 16: return launch_one<EPI, 16>(p, num_sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -848,43 +769,6 @@ cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, i
              : launch_rank<EPI_SWIGLU>(p13, a.lrank, num_sms, s);
   if (e != cudaSuccess || !(stages & 2)) return e;
   return pair ? launch_pair<EPI_F32>(p2, num_sms, s) : launch_rank<EPI_F32>(p2, a.lrank, num_sms, s);
-}
-
-cudaError_t launch_lora_down_tc(const FfnArgs& a, const void* xp, int mcap, int num_sms,
-                                cudaStream_t s, int stage) {
-  TcParams p;
-  memset(&p, 0, sizeof(p));
-  const size_t d = size_t(a.d), w = size_t(a.w);
-  const int r = a.lrank;
-  if (r != 8 && r != 16) return cudaErrorInvalidValue;
-  const bool s13 = stage == 1;
-  const size_t K = s13 ? d : w;
-  if (!encode_2d(&p.tma_a, s13 ? xp : a.h, K, size_t(mcap))) return cudaErrorInvalidValue;
-  const LoraOffsets lo = lora_offsets(a.d, a.w, r);
-  for (int sgi = 0; sgi < a.nseg; ++sgi) {
-    const char* blk = reinterpret_cast<const char*>(a.lblk[sgi]);
-    if (!blk) continue;  // no adapter: the tile is skipped (its U rows are never read)
-    const bool ok = s13 ? encode_adapter_a13(&p.tma_b[sgi], blk, d, uint32_t(r), lo.a3)
-                        : encode_adapter_a2(&p.tma_b[sgi], blk + lo.a2 * 2, w, uint32_t(r));
-    if (!ok) return cudaErrorInvalidValue;
-    p.wmask[sgi >> 5] |= 1u << (sgi & 31);
-  }
-  p.off = a.off;
-  p.hdr = a.hdr;
-  p.err = a.err;
-  p.nseg = a.nseg;
-  p.b3d = s13 ? 1 : 0;
-  p.out = const_cast<float*>(s13 ? a.u13 : a.u2);  // bf16 [rows, 2r] / [rows, r]
-  p.lscale = a.lscale;
-  p.kblocks = int(K / BK);
-  p.ntiles_n = 1;
-  p.ldo = s13 ? 2 * r : r;
-  p.group_m = 1;
-  const int mtiles = (mcap + BM - 1) / BM;
-  const int grid = mtiles < num_sms ? (mtiles > 0 ? mtiles : 1) : num_sms;
-  // N = 2r for [A1; A3]; 16 for A2 (r = 8: rows 8-15 of the box are zero)
-  return s13 && r == 16 ? launch_one<EPI_DOWN, 0, 32>(p, grid, s)
-                        : launch_one<EPI_DOWN, 0, 16>(p, grid, s);
 }
 
 }  // namespace mcft

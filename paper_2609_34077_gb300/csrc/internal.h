@@ -280,12 +280,6 @@ bool tc_pair_tiles(int T, int K, int E, int lrank);
 // split: bf16 halves of the LoRA middle vectors (u13 / u2 as launch_lora_down_tiles wrote them).
 cudaError_t launch_ffn_rows(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s,
                             int stages, int split);
-// Down projections of the adapters for the tcgen05 path, on the tensor cores, bf16 out scaled by
-// s: stage 1: u13[q] = s [A1 xp[q] | A3 xp[q]] (N = 2r); stage 2: u2[q] = s A2 h[q] (N = 16),
-// for the rows of every segment with an adapter. The expert GEMMs add the up projections.
-cudaError_t launch_lora_down_tc(const FfnArgs& a, const void* xp, int mcap, int num_sms,
-                                cudaStream_t s, int stage);
-
 struct CombineArgs {
   const float* o;
   const float* gate;
