@@ -542,14 +542,20 @@ __device__ bool wait_landed(const FfnArgs& a, unsigned epoch, int e, size_t off,
 // missed expert waits (bounded) for the stamps of the pieces it reads. Those waits end too: a CTA
 // that holds an FFN item took its role after the a.nfetch fetchers took theirs, so every fetcher
 // is running, and fetchers wait on nothing until all pieces are copied.
-// FETCH: the build for launches that fetch their own misses (a.nfetch > 0); the plain build
-// carries none of that code.
-template <int MAXNG, bool FETCH>
-__global__ void __launch_bounds__(kWarps * 32, 2)
-    dec_fused_kernel(const __grid_constant__ FfnArgs a, int RB13, int RB2) {
+// Builds: kPlain; kFetch for launches that fetch their own misses (a.nfetch > 0; the plain build carries
+// none of that code); and dec_beside_kernel, for launches of one or two tokens that run beside a fetch
+// kernel. Two CTAs of 256 threads at up to 128 registers fill an SM, so a fetch kernel needs slots kept
+// free for it; up to 8 tokens also fit 96 registers without spills, which leaves room for one of its
+// 40-register CTAs beside two of these, so that build takes every slot. Three-layer DeepSeek-V2-Lite
+// chain with prefetch 2: T = 1 206 -> 198 us, T = 2 297 -> 290, but T = 4, which the link bounds, 857 / 864.
+// Alone 96 registers are slower (T = 1 44.1 / 44.7 us, a chain without prefetch 157 / 162).
+enum { kPlain = 0, kFetch = 1 };
+constexpr int kBesideMaxT = 2;
+template <int MAXNG, int BUILD>
+__device__ __forceinline__ void dec_fused(const FfnArgs& a, int RB13, int RB2) {
   // fetching and streaming are compiled into the kernels of up to kStreamMaxT tokens (the host
   // only asks for them there)
-  constexpr bool kStreams = FETCH && 8 * MAXNG <= kStreamMaxT;
+  constexpr bool kStreams = BUILD == kFetch && 8 * MAXNG <= kStreamMaxT;
   __shared__ DecItems it13, it2;
   __shared__ float red[kWarps * kMaxNG * 8 * 32];
   __shared__ int s_next, s_ok, s_role;
@@ -663,6 +669,17 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
   }
 }
 
+template <int MAXNG, int BUILD>
+__global__ void __launch_bounds__(kWarps * 32, 2)
+    dec_fused_kernel(const __grid_constant__ FfnArgs a, int RB13, int RB2) {
+  dec_fused<MAXNG, BUILD>(a, RB13, RB2);
+}
+
+__global__ void __maxnreg__(96)
+    dec_beside_kernel(const __grid_constant__ FfnArgs a, int RB13, int RB2) {
+  dec_fused<1, kPlain>(a, RB13, RB2);
+}
+
 int blocks_per_sm(const void* fn) {
   int nb = 1;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kWarps * 32, 0) != cudaSuccess || nb < 1)
@@ -724,19 +741,27 @@ cudaError_t launch_decode_ng(const FfnArgs& a, int num_sms, cudaStream_t s, int 
   if (stages == 3 && a.done && a.lrank == 0) {
     // both GEMMs in one launch with claimed items
     static const int nbf =
-        blocks_per_sm(reinterpret_cast<const void*>(dec_fused_kernel<MAXNG, false>));
+        blocks_per_sm(reinterpret_cast<const void*>(dec_fused_kernel<MAXNG, kPlain>));
     const int gf = max(num_sms, num_sms * nbf - reserved);
+    if constexpr (MAXNG == 1) {
+      if (reserved > 0 && a.nfetch == 0 && a.T <= kBesideMaxT) {
+        prof_begin(kProfDecFused, s);
+        e = launch_pdl(dec_beside_kernel, dim3(num_sms * 2), dim3(kWarps * 32), 0, s, a, rb13, rb2);
+        prof_end(kProfDecFused, s);
+        return e != cudaSuccess ? e : cudaGetLastError();
+      }
+    }
     if constexpr (8 * MAXNG <= kStreamMaxT) {
       if (a.nfetch > 0) {  // fetching its own misses
         prof_begin(kProfDecFetch, s);
-        e = launch_pdl(dec_fused_kernel<MAXNG, true>, dim3(gf), dim3(kWarps * 32), 0, s, a, rb13,
+        e = launch_pdl(dec_fused_kernel<MAXNG, kFetch>, dim3(gf), dim3(kWarps * 32), 0, s, a, rb13,
                        rb2);
         prof_end(kProfDecFetch, s);
         return e != cudaSuccess ? e : cudaGetLastError();
       }
     }
     prof_begin(kProfDecFused, s);
-    e = launch_pdl(dec_fused_kernel<MAXNG, false>, dim3(gf), dim3(kWarps * 32), 0, s, a, rb13, rb2);
+    e = launch_pdl(dec_fused_kernel<MAXNG, kPlain>, dim3(gf), dim3(kWarps * 32), 0, s, a, rb13, rb2);
     prof_end(kProfDecFused, s);
     return e != cudaSuccess ? e : cudaGetLastError();
   }
