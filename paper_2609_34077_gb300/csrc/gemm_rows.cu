@@ -24,7 +24,7 @@
 // * DeepSeek-V2-Lite shape, 4096 tokens on 48 of 64 experts (512 rows each): GEMM13 355 -> 274 us
 //   (1.38 PFLOP/s), GEMM2 184 -> 166 us (1.14). The old tiles paid 12 % for padding and read 1.28 GB of
 //   DRAM where 0.69 GB does. Now the MMAs run 66 % of the cycles at about 1.85 GHz under the power
-//   cap; wider rounds, weights prefetched into L2 and narrower token tiles were all slower.
+//   cap; narrower token tiles and weights prefetched into L2 were slower.
 // * 200 tokens (19 rows an expert): HBM, the weights read once: GEMM13 145 -> 106 us (7.2 TB/s, the h
 //   rows included), GEMM2 68 -> 61 us.
 // * Mixtral shape, 4096 tokens (2048 rows an expert), GEMM13 1254 -> 1206 us, GEMM2 650 -> 703 us: the
