@@ -21,14 +21,20 @@
 // apart, and meet with one shuffle per pair of columns.
 //
 // What bounds it (GB300, CUDA events in a steady loop, against the 128-row tiles of gemm_tc.cu):
-// * DeepSeek-V2-Lite shape, 4096 tokens on 48 of 64 experts (512 rows each): GEMM13 355 -> 274 us
-//   (1.38 PFLOP/s), GEMM2 184 -> 166 us (1.14). The old tiles paid 12 % for padding and read 1.28 GB of
-//   DRAM where 0.69 GB does. Now the MMAs run 66 % of the cycles at about 1.85 GHz under the power
-//   cap; narrower token tiles and weights prefetched into L2 were slower.
-// * 200 tokens (19 rows an expert): HBM, the weights read once: GEMM13 145 -> 106 us (7.2 TB/s, the h
-//   rows included), GEMM2 68 -> 61 us.
-// * Mixtral shape, 4096 tokens (2048 rows an expert), GEMM13 1254 -> 1206 us, GEMM2 650 -> 703 us: the
-//   power cap bounds both, and there gemm_tc.cu keeps the large segments (see ws_layout).
+// * DeepSeek-V2-Lite shape, 4096 tokens on 48 of 64 experts (512 rows each): GEMM13 355 -> 240 us
+//   (1.57 PFLOP/s), GEMM2 184 -> 154 us (1.23): the MMAs and the power cap. The old tiles paid 12 % for
+//   padding and read 1.28 GB of DRAM where 0.69 GB does. Narrower token tiles and weights prefetched
+//   into L2 were slower.
+// * 200 tokens (19 rows an expert): HBM, the weights read once: GEMM13 145 -> 100 us, GEMM2 68 -> 56 us
+//   (525 and 264 MB of weights: 5.3 and 4.7 TB/s, the start and the last round of tiles included).
+// * Mixtral shape, 4096 tokens (2048 rows an expert), GEMM13 1219 -> 1147 us, GEMM2 661 -> 637 us: the
+//   power cap.
+// The two threads that issue are what the loops wait for when they are not kept short: with the ring
+// walked under a lane test (operands moved to uniform registers one by one), tokens fetched as up to
+// four boxes and the peer's barrier address found per block, the rates above were GEMM13 300 and
+// GEMM2 175 us at 4096 DeepSeek tokens, 106 and 61 us at 200. One elected lane, one box per half tile
+// (hence a map for each size) and the addresses found once per tile gave the rest. Two k-blocks per
+// stage and per copy (5-D and 3-D boxes) were faster than the old loop and are slower than this one.
 // Eight epilogue warps rather than four, and a quotient without branches (silu_to_bf16): the SwiGLU of a
 // tile took about 28,000 cycles on four warps, more than the MMAs of a 2048-long contraction (16,400).
 // d = 960, w = 704 (15 k-blocks), 16 experts: GEMM13 at T = 4096 99 -> 63 us by the quotient alone.
@@ -58,7 +64,8 @@ constexpr int kEpiGroups = 2;                 // of four warps, one per TMEM lan
 constexpr int kThreads = 64 + kEpiGroups * 128;
 constexpr int BK = 64;
 constexpr int kTileTok = 256;                 // most tokens of a tile
-constexpr int kBoxes = 4;                     // token boxes of 16, 32, 64 and 128 rows
+constexpr int kBoxes = 8;                     // token boxes of 16, 32, .. 128 rows: one per half tile
+constexpr int kUBoxes = 4;                    // adapters' U: boxes of 16, 32, 64 and 128 rows, combined
 constexpr int kMaxStages = 10;
 constexpr int kABytes = 128 * BK * 2;         // a CTA's weight rows of a stage
 constexpr int kRingBytes = 6 * (kABytes + (kTileTok / 2) * BK * 2);
@@ -74,7 +81,7 @@ constexpr int kStgBytes = 32 * kStgRow;
 enum { EPI_SWIGLU = 0, EPI_F32 = 1 };
 
 struct RowsParams {
-  CUtensorMap x[kBoxes];   // permuted rows (GEMM13: gathered x; GEMM2: h), boxes of 16 << i rows
+  CUtensorMap x[kBoxes];   // permuted rows (GEMM13: gathered x; GEMM2: h), boxes of 16 (i + 1) rows
   CUtensorMap sx[kBoxes];  // GEMM13: x itself, whose rows are the shared experts' rows in order
   CUtensorMap w[kMaxSeg];
   const int* off;
@@ -85,11 +92,13 @@ struct RowsParams {
   int nseg, E, kblocks, mtiles, ldo, group_x, use_sx;
 };
 struct RowsLoraParams : RowsParams {
-  CUtensorMap u[kMaxExtra][kBoxes];  // U of each extra k-block
+  CUtensorMap u[kMaxExtra][kUBoxes];  // U of each extra k-block
   CUtensorMap lb[2][kMaxSeg];        // GEMM13: B1, B3; GEMM2: B2
   uint32_t lmask[3];                 // segments with an adapter
   int nx;
 };
+
+static_assert(sizeof(RowsLoraParams) <= 32764, "kernel parameters");
 
 struct Ctl {
   uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
@@ -278,50 +287,60 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   };
 
   if (warp == 0) {
-    if (lane == 0 && cid < tiles) {
+    if (cid < tiles && elect_one()) {
+      const uint32_t fb0 = peer_addr(&ctl->full[0], 0);
       int s = 0, issued = 0;
       uint32_t ph = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
         const TileAt t = tile_at(ctl, nseg, p.mtiles, p.group_x, tile);
-        const int half = t.cols() / 2;
+        const int half = t.cols() / 2, mrow = t.mt * 2 + int(rank);
         const bool sx = EPI == EPI_SWIGLU && p.use_sx && t.seg >= p.E;
         const int xrow = t.row0 - (sx ? ctl->off[t.seg] : 0) + int(rank) * half;
-        const int urow = t.row0 + int(rank) * half;
-        const int nkb = p.kblocks + extra_of(t.seg);
         const uint32_t bytes = 2u * uint32_t(kABytes + half * BK * 2);
-        for (int kb = 0; kb < nkb; ++kb) {
+        const CUtensorMap* mw = &p.w[t.seg];
+        const CUtensorMap* mx = (sx ? p.sx : p.x) + (half / 16 - 1);
+        const int nkb = p.kblocks;
+        int kb = 0;
+        for (; kb < nkb; ++kb) {
           if (!mbar_wait_cl(&ctl->empty[s], ph ^ 1u, abort, p.err)) break;
-          const uint32_t sa = base + uint32_t(s * stage_bytes), sb = sa + kABytes;
-          const uint32_t fb = peer_addr(&ctl->full[s], 0);
+          const uint32_t sa = base + uint32_t(s * stage_bytes), fb = fb0 + uint32_t(s) * 8u;
           if (leader) mbar_expect_tx(&ctl->full[s], bytes);
-          const CUtensorMap* mw = &p.w[t.seg];
-          const CUtensorMap* mx = sx ? p.sx : p.x;
-          int c0 = kb * BK, plane = 0, row = xrow;
-          if constexpr (LORA) {
-            if (kb >= p.kblocks) {
-              const int e = kb - p.kblocks, m = EPI == EPI_SWIGLU ? (e & 1) : 0;
-              mw = &p.lb[m][t.seg];
-              mx = p.u[e];
-              c0 = 0;
-              plane = -m;  // B1 fills the gate rows of the box, B3 (entered at -1) the up rows
-              row = urow;
-            }
-          }
           if constexpr (EPI == EPI_SWIGLU)
-            tma_load_4d_pair(sa, mw, c0, 0, plane, (t.mt * 2 + int(rank)) * 4, fb);
+            tma_load_4d_pair(sa, mw, kb * BK, 0, 0, mrow * 4, fb);
           else
-            tma_load_2d_pair(sa, mw, c0, t.mt * 256 + int(rank) * 128, fb);
-          int r = 0;
-#pragma unroll
-          for (int b = kBoxes - 1; b >= 0; --b)
-            if (half & (16 << b)) {
-              tma_load_2d_pair(sb + uint32_t(r) * (BK * 2), mx + b, c0, row + r, fb);
-              r += 16 << b;
-            }
+            tma_load_2d_pair(sa, mw, kb * BK, mrow * 128, fb);
+          tma_load_2d_pair(sa + kABytes, mx, kb * BK, xrow, fb);
           if (issued < stages) ++issued;
           if (++s == stages) {
             s = 0;
             ph ^= 1u;
+          }
+        }
+        if constexpr (LORA) {
+          const int nx = kb == nkb ? extra_of(t.seg) : 0;
+          for (int e = 0; e < nx; ++e) {
+            if (!mbar_wait_cl(&ctl->empty[s], ph ^ 1u, abort, p.err)) break;
+            const uint32_t sa = base + uint32_t(s * stage_bytes), fb = fb0 + uint32_t(s) * 8u;
+            if (leader) mbar_expect_tx(&ctl->full[s], bytes);
+            // B1 fills the gate rows of the box, B3 (entered at plane -1) the up rows
+            const int m = EPI == EPI_SWIGLU ? (e & 1) : 0;
+            if constexpr (EPI == EPI_SWIGLU)
+              tma_load_4d_pair(sa, &p.lb[m][t.seg], 0, 0, -m, mrow * 4, fb);
+            else
+              tma_load_2d_pair(sa, &p.lb[m][t.seg], 0, mrow * 128, fb);
+            int r = 0;
+#pragma unroll
+            for (int b = kUBoxes - 1; b >= 0; --b)
+              if (half & (16 << b)) {
+                tma_load_2d_pair(sa + kABytes + uint32_t(r) * (BK * 2), &p.u[e][b], 0,
+                                 t.row0 + int(rank) * half + r, fb);
+                r += 16 << b;
+              }
+            if (issued < stages) ++issued;
+            if (++s == stages) {
+              s = 0;
+              ph ^= 1u;
+            }
           }
         }
       }
@@ -335,7 +354,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (leader && lane == 0 && cid < tiles) {
+    if (leader && cid < tiles && elect_one()) {
       int s = 0;
       uint32_t ph = 0, lt = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
@@ -468,7 +487,7 @@ bool encode_rows(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows,
 }
 bool encode_boxes(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows, uint64_t stride) {
   for (int b = 0; b < kBoxes; ++b)
-    if (!encode_rows(m + b, base, cols, rows, stride, 16u << b)) return false;
+    if (!encode_rows(m + b, base, cols, rows, stride, 16u * uint32_t(b + 1))) return false;
   return true;
 }
 // Rows of `planes` matrices [rows, cols] (plane stride in elements), interleaved 16 by 16: box of 64
@@ -551,7 +570,9 @@ bool fill_lora(RowsLoraParams& p, const FfnArgs& a, int mcap, int stage, int spl
   p.nx = (stage == 1 ? 2 : 1) * split;
   const char* u = reinterpret_cast<const char*>(stage == 1 ? a.u13 : a.u2);
   for (int e = 0; e < p.nx; ++e)
-    if (!encode_boxes(p.u[e], u + size_t(e) * r * 2, r, uint64_t(mcap), p.nx * r)) return false;
+    for (int b = 0; b < kUBoxes; ++b)
+      if (!encode_rows(&p.u[e][b], u + size_t(e) * r * 2, r, uint64_t(mcap), p.nx * r, 16u << b))
+        return false;
   for (int s = 0; s < a.nseg; ++s) {
     const char* blk = reinterpret_cast<const char*>(a.lblk[s]);
     if (!blk || !a.wblk[s]) continue;
