@@ -470,18 +470,15 @@ mcft_status mcft_test_inject(int fail_pinned_allocs, int fail_expert_copies,
  * workspace, so set it before sizing workspaces (mcft_moe_workspace_size) and keep it while they
  * are in use: a workspace sized under one setting may be too small under the other, which the
  * forward then rejects with MCFT_ERR_INVALID.
- *   MCFT_TC_TILES_ONE_CTA   (default) chosen by size: 128 x 256 tiles, one CTA per SM, segments
- *                           padded to 128 rows, for layers with d and w of at least 4096 (and
- *                           multiples of 256 and 128) whose routed experts average at least 768
- *                           rows; else 256 weight rows x up to 256 tokens on pairs of CTAs, segments
- *                           unpadded;
- *   MCFT_TC_TILES_CTA_PAIR  256 x 256 tiles on pairs of CTAs (cta_group::2 MMAs issued by one CTA
+ *   MCFT_TC_TILES_ONE_CTA   (default; the name is that of an earlier kernel) 256 weight rows x up to
+ *                           256 tokens on pairs of CTAs, segments unpadded;
+ *   MCFT_TC_TILES_CTA_PAIR  256 tokens x 256 weight rows on pairs of CTAs (cta_group::2 MMAs issued by one CTA
  *                           of a 2-CTA cluster over both CTAs' shared memory), segments padded to
  *                           256 rows, for layers without adapters whose routed experts average at
- *                           least 512 rows (others keep the one-CTA tiles). Each output is the
+ *                           least 512 rows (others keep the default tiles). Each output is the
  *                           same products summed in the same order; on every shape tested the
- *                           outputs equal the one-CTA tiles' bit for bit. Slower than the one-CTA
- *                           tiles on the GB300 shapes measured (kept for comparison).
+ *                           outputs equal the default tiles' bit for bit. Slower than the default
+ *                           on the GB300 shapes measured (kept for comparison).
  * MCFT_ERR_INVALID for another mode. */
 typedef enum { MCFT_TC_TILES_ONE_CTA = 0, MCFT_TC_TILES_CTA_PAIR = 1 } mcft_tc_tiles;
 mcft_status mcft_set_tc_tiles(int mode);

@@ -151,17 +151,14 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   L.ks = L.decode ? decode_ksplit(T) : 1;
   const bool pair = L.tc && aligned && g_tc_tiles.load() == MCFT_TC_TILES_CTA_PAIR &&
                     tc_pair_tiles(T, K, E, lrank);
-  // The 128-row tiles of gemm_tc.cu keep the layers whose contractions are long and whose experts
-  // average many rows; everything else runs with the weight rows on M (gemm_rows.cu). Whole passes,
-  // gemm_tc against gemm_rows: Mixtral shape at T = 4096 (1024 rows by T K / E) 1978 / 2028 us and at
-  // 8192 3760 / 3977, but 928 / 792 at 1500 (375 rows) and at 3000 (750) even, 1496 / 1519;
-  // DeepSeek-V2-Lite shape (contractions of 2048 and 1408) 641 / 540 at 4096, 2112 / 1908 at 16384
-  // (1536 rows). The choice must not depend on adapters: mcft_gate_grad reads the workspace of a
-  // forward without knowing whether it had any.
-  const bool big = aligned && d >= 4096 && w >= 4096 && size_t(T) * K >= size_t(768) * E;
-  L.rows = L.tc && !pair && !big;
+  // The weight rows on M (gemm_rows.cu) unless the 256-row token tiles were asked for (gemm_tc.cu).
+  // Whole passes, 128-row token tiles (removed) against gemm_rows: Mixtral shape at T = 2000 953 / 952
+  // us, 4096 1940 / 1875, 8192 3753 / 3675, all 8 experts kept at 4096 2080 / 1947; DeepSeek-V2-Lite
+  // shape at 4096 641 / 478. The choice must not depend on adapters: mcft_gate_grad reads the
+  // workspace of a forward without knowing whether it had any.
+  L.rows = L.tc && !pair;
   L.split = aligned ? 1 : 2;
-  L.pad = pair ? 256 : L.tc && !L.rows ? 128 : 1;
+  L.pad = pair ? 256 : 1;
   const int nseg = E + S;
   L.mcap = T * K + S * T + nseg * (L.pad - 1);
   size_t o = 0;

@@ -20,7 +20,8 @@
 // same outputs, so the gate and up values of an output sit in one warp's TMEM quarter, 16 lanes
 // apart, and meet with one shuffle per pair of columns.
 //
-// What bounds it (GB300, CUDA events in a steady loop, against the 128-row tiles of gemm_tc.cu):
+// What bounds it (GB300, CUDA events in a steady loop, against 128-row token tiles with the
+// tokens on M, since removed):
 // * DeepSeek-V2-Lite shape, 4096 tokens on 48 of 64 experts (512 rows each): GEMM13 355 -> 240 us
 //   (1.57 PFLOP/s), GEMM2 184 -> 154 us (1.23): the MMAs and the power cap. The old tiles paid 12 % for
 //   padding and read 1.28 GB of DRAM where 0.69 GB does. Narrower token tiles and weights prefetched

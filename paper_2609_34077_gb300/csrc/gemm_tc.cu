@@ -1,30 +1,33 @@
-// Grouped expert GEMMs on the 5th-generation tensor cores (tcgen05 + TMEM), fed by TMA.
+// Grouped expert GEMMs with the tokens on the MMA's M side, on CTA pairs (tcgen05 + TMEM, fed by TMA):
+// the tile shape that mcft_set_tc_tiles(MCFT_TC_TILES_CTA_PAIR) selects. The default is gemm_rows.cu.
 //
 // Section 3.1: each routed expert is F(x) = W2 (silu(W1 x) * (W3 x)) (SwiGLU); with tokens
-// permuted into per-expert segments (padded to 128 rows), the two expert GEMMs of a layer are
+// permuted into per-expert segments (padded to 256 rows), the two expert GEMMs of a layer are
 //   GEMM13: acc[m, 0:128] = xp[m] . W1[n0:n0+128]^T, acc[m, 128:256] = xp[m] . W3[n0:n0+128]^T,
 //           h[m, n0:n0+128] = bf16(silu(acc_gate) * acc_up)             (fused epilogue)
 //   GEMM2:  o[m, n0:n0+256] = h[m] . W2[n0:n0+256]^T                       (fp32 out)
 // both D = A B^T with A and B K-major bf16, fp32 accumulators in tensor memory.
-// With LoRA adapters (Section 3.2, Stage 2) every projection is W v + s B (A v). The down projections
-// U13[m] = s [A1 xp[m] | A3 xp[m]] and U2[m] = s A2 h[m] come from lora.cu in bf16, and the up
-// projections ride on the expert GEMMs as one extra k-block per adapted tile,
-// D += U B'^T, so the tensor cores add them to the accumulators and the epilogues are unchanged.
 //
-// One persistent CTA per SM, 6 warps (7 with adapters):
-//   warp 0  - TMA producer (one thread): A tile 128x64 and B tile 256x64 per stage, 4 stages,
-//             128-byte swizzle, one mbarrier with a transaction count per stage;
-//   warp 1  - allocates 512 TMEM columns (two 128x256 fp32 accumulators) and issues
-//             tcgen05.mma (M=128, N=256, K=16) from one thread; tcgen05.commit frees a stage /
-//             publishes an accumulator;
-//   warps 2-5 - epilogue: tcgen05.ld of their 32-lane quarter, SwiGLU or fp32, staged through
-//             shared memory and stored as whole 128-byte row segments; they release the
-//             accumulator so the next tile's MMAs overlap this tile's epilogue;
-//   warp 6  - with adapters only: writes each adapted tile's extra k-block (see LoraOps).
-// Tiles are walked m-fastest inside groups of m-tiles so concurrently running CTAs share weight
+// Tiles of 256 rows x 256 columns, one MMA of M = 256 per K step issued by the pair's leader over both
+// CTAs' shared memory. Each CTA loads its 128 activation rows and its half of the tile's 256 weight
+// rows (GEMM13: rank 0 the W1 rows, rank 1 the W3 rows, i.e. the gate and up halves of N; GEMM2: 128
+// consecutive W2 rows each), so every weight element is read from shared memory once for the rows of
+// both CTAs. 6 stages of 32 KB:
+//   warp 0 (both CTAs) - TMA producer (one thread); the loads of both CTAs complete on the leader's
+//             full[s], on which the leader expects the pair's bytes; each CTA waits on its own empty[s];
+//   warp 1 - allocates the pair's TMEM (both CTAs), two 128 x 256 fp32 accumulators each; in the
+//             leader, issues the MMAs, whose commits arrive on empty[s] and tfull[b] of both CTAs;
+//   warps 2-5 (both CTAs) - epilogue of the CTA's 128 rows of the tile: tcgen05.ld of their 32-lane
+//             quarter, SwiGLU or fp32, staged through shared memory and stored as whole 128-byte row
+//             segments; they release the accumulator on the leader's tempty[b] (eight arrivals: four
+//             warps per CTA), so the next tile's MMAs overlap this tile's epilogue.
+// Tiles are walked m-fastest inside groups of m-tiles so concurrently running pairs share weight
 // tiles (and the activation group) in L2. Every wait is bounded: after 2 s the kernel records
 // MCFT_ERR_TIMEOUT, stops issuing, waits (bounded) for its copies and MMAs in flight, frees TMEM
-// and returns.
+// and returns. The leader drains its last stages' copies (both CTAs' bytes), the peer waits (bounded)
+// until its last stages were consumed, and both CTAs leave through one cluster barrier after the
+// leader's MMAs have completed, so neither exits while the other may still read its shared memory or
+// arrive on its barriers.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -37,10 +40,15 @@ namespace {
 
 constexpr int BM = 128, BN = 256, BK = 64;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int kMaxStages = 6;  // of the pair tiles
+constexpr int kPairRows = 2 * BM;
+constexpr int kPairStages = 6;
+constexpr int kPairStageBytes = A_BYTES + (BN / 2) * BK * 2;  // 128 activation + 128 weight rows
+constexpr int kPairTmemCols = 2 * BN;                          // two 128 x 256 accumulators
+// Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A bf16 (bits 7-9 = 1), B bf16
+// (bits 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
+constexpr uint32_t kPairIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) |
+                                (uint32_t(kPairRows >> 4) << 24);
 constexpr int kThreads = 192;  // producer, MMA, 4 epilogue warps
-constexpr int kBuilderWarp = 6;  // with adapters: one more warp writes the extra k-blocks
-__host__ __device__ constexpr int threads_for(int lr) { return lr > 0 ? kThreads + 32 : kThreads; }
 
 enum { EPI_SWIGLU = 0, EPI_F32 = 1 };
 
@@ -53,17 +61,10 @@ struct TcParams {
   unsigned* err;
   uint32_t wmask[3];  // segments that have weights
   int nseg, kblocks, ntiles_n, ldo, b_half, group_m;
-  // LoRA (Stage 2): adapter block per segment (NULL: none); lug: the U operand rows (bf16;
-  // GEMM13 [rows, 2r] = s [A1 x | A3 x], GEMM2 [rows, r] = s A2 h); lb0 / lb1: element offsets
-  // of the up matrices (B1, B3 for GEMM13; B2 for GEMM2).
-  const char* lblk[kMaxSeg];
-  const uint16_t* lug;
-  size_t lb0, lb1;
 };
 
 struct SmemCtl {
-  uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
-  uint64_t bgo[2];  // with adapters: the producer hands the extra k-blocks' stages to the builder
+  uint64_t full[kPairStages], empty[kPairStages], tfull[2], tempty[2], drain;
   uint32_t tmem_base;
   int abort;
   int mt_total;
@@ -71,28 +72,14 @@ struct SmemCtl {
   int off[kMaxSeg + 1];
 };
 
-// Geometry: 4 stages of 48 KB, two 128 x 256 fp32 accumulators = all 512 TMEM columns.
 // Epilogue store staging: each epilogue warp writes 32 rows x 128 bytes of its
 // output into shared memory (rows padded to 144 bytes: conflict-free 16-byte writes and reads),
 // then stores them as whole 128-byte row segments, four rows per instruction.
 constexpr int kOutRowBytes = 144;
 constexpr int kOutWarpBytes = 32 * kOutRowBytes;
 constexpr int kCtlBytes = (int(sizeof(SmemCtl)) + 15) / 16 * 16;
-
-struct Tile {
-  static constexpr int NB = BN;
-  static constexpr int B_BYTES = NB * BK * 2;
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int STAGES = 4;
-  static constexpr int TMEM_COLS = 2 * NB;
-  // Instruction descriptor, kind::f16: D fp32 (bits 4-5 = 1), A bf16 (bits 7-9 = 1), B bf16
-  // (bits 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
-  static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) |
-                                    (uint32_t(NB >> 3) << 17) | (uint32_t(BM >> 4) << 24);
-  static constexpr int OUT_STAGE = 4 * kOutWarpBytes;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + kCtlBytes + OUT_STAGE;
-  static_assert(SMEM <= 227 * 1024, "shared memory");
-};
+constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + kCtlBytes + 4 * kOutWarpBytes;
+static_assert(kPairSmem <= 227 * 1024, "shared memory");
 
 // Tile -> (m-tile, n-tile): groups of group_m m-tiles; inside a group, n-major then m.
 __device__ __forceinline__ void tile_coords(int tile, int mt_total, int ntn, int G, int& mt,
@@ -109,77 +96,6 @@ __device__ __forceinline__ int seg_of_row(const SmemCtl* c, int row) {
   while (s + 1 < c->nseg && c->off[s + 1] <= row) ++s;
   return s;
 }
-
-// The adapter operands of the extra k-block an adapted tile appends to its K loop (the up
-// projections on the tensor cores): D += U B'^T with
-//   GEMM13: U = [s A1 x | s A3 x] (K' = 2r), B' = [B1 rows | 0] for the gate half and
-//           [0 | B3 rows] for the up half (block-diagonal, so one pass of N = 256 adds both);
-//   GEMM2:  U = [s A2 h | 0], B' = [B2 rows | 0] (K' = r, zero-padded to 16).
-// U and the B rows are bf16 in global memory (U written by the down-projection kernel / by
-// GEMM13). The producer warp loads them into registers when it starts the tile, and writes them
-// into the stage's A and B regions in the 128-byte-swizzled K-major layout the TMA tiles use
-// (16-byte chunk c of row i at chunk c ^ (i % 8) of the row's 128 bytes) when the extra k-block's
-// stage is free. Only the first K' columns of the stage are written and read.
-template <int EPI, int LR>
-struct LoraOps {
-  static constexpr int KL = EPI == EPI_SWIGLU ? 2 * LR : (LR < 16 ? 16 : LR);  // K' of the block
-  static constexpr int UC = (EPI == EPI_SWIGLU ? 2 * LR : LR) / 8;  // data chunks of a U row
-  static constexpr int BC = LR / 8;                                 // data chunks of a B row
-  static constexpr int CH = KL / 8;                                 // chunks written per row
-  uint4 u[4][UC];  // tile rows 4 lane + i
-  uint4 b[8][BC];  // B' rows lane + 32 i
-
-  __device__ __forceinline__ void load(const TcParams& p, const char* lb, int mt, int nt,
-                                       int lane) {
-    const int ucols = EPI == EPI_SWIGLU ? 2 * LR : LR;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint4* src =
-          reinterpret_cast<const uint4*>(p.lug + (size_t(mt) * BM + 4 * lane + i) * ucols);
-#pragma unroll
-      for (int c = 0; c < UC; ++c) u[i][c] = __ldcg(src + c);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int j = lane + 32 * i;
-      size_t el;
-      if constexpr (EPI == EPI_SWIGLU)
-        el = j < BN / 2 ? p.lb0 + (size_t(nt) * (BN / 2) + j) * LR
-                        : p.lb1 + (size_t(nt) * (BN / 2) + j - BN / 2) * LR;
-      else
-        el = p.lb0 + (size_t(nt) * BN + j) * LR;
-      const uint4* src = reinterpret_cast<const uint4*>(lb + el * 2);
-#pragma unroll
-      for (int c = 0; c < BC; ++c) b[i][c] = __ldg(src + c);
-    }
-  }
-
-  __device__ __forceinline__ void store(uint8_t* sa, uint8_t* sb, int lane) const {
-    const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int row = 4 * lane + i;
-      uint4* dst = reinterpret_cast<uint4*>(sa + row * 128);
-#pragma unroll
-      for (int c = 0; c < CH; ++c) dst[c ^ (row & 7)] = c < UC ? u[i][c] : z;
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int row = lane + 32 * i;
-      uint4* dst = reinterpret_cast<uint4*>(sb + row * 128);
-      // GEMM13: gate rows hold B1 in chunks [0, BC), up rows B3 in chunks [BC, 2 BC)
-      const int c0 = EPI == EPI_SWIGLU && row >= BN / 2 ? BC : 0;  // i >= 4: known when unrolled
-#pragma unroll
-      for (int c = 0; c < CH; ++c) {
-        uint4 v = z;
-#pragma unroll
-        for (int e = 0; e < BC; ++e)
-          if (c == c0 + e) v = b[i][e];
-        dst[c ^ (row & 7)] = v;
-      }
-    }
-  }
-};
 
 // Epilogue of one expert-GEMM tile for the 32 accumulator rows of an epilogue warp (TMEM lane
 // quarter at taddr, output rows grow0 .. grow0 + 31, n-tile nt): SwiGLU to bf16 h (GEMM13) or fp32
@@ -242,238 +158,6 @@ __device__ __forceinline__ void store_tile(const TcParams& p, uint8_t* stg, uint
   }
 }
 
-template <int EPI, int LR>
-__global__ void __launch_bounds__(threads_for(LR), 1) gemm_tc_kernel(const __grid_constant__ TcParams p) {
-  using C = Tile;
-  constexpr int NB = C::NB;
-  constexpr int STAGES = C::STAGES, STAGE_BYTES = C::STAGE_BYTES, TMEM_COLS = C::TMEM_COLS;
-  constexpr int LRA = LR > 0 ? LR : 8;
-  using LOps = LoraOps<EPI, LRA>;
-  pdl_wait();
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  SmemCtl* ctl = reinterpret_cast<SmemCtl*>(smem_raw + (base - raw) + STAGES * STAGE_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-  if (threadIdx.x == 0) {
-    int abort = p.hdr->abort;
-    const int nseg = p.nseg;
-    ctl->nseg = nseg;
-    for (int s = 0; s <= nseg; ++s) ctl->off[s] = p.off[s];
-    for (int s = 0; s < nseg; ++s) {
-      if (ctl->off[s + 1] > ctl->off[s] && !((p.wmask[s >> 5] >> (s & 31)) & 1u)) {
-        set_error(p.err, kErrInvalid);  // a selected expert without weights
-        const_cast<WsHeader*>(p.hdr)->abort = 1;  // later kernels of the call skip their work
-        abort = 1;
-      }
-    }
-    ctl->abort = abort;
-    ctl->mt_total = abort ? 0 : ctl->off[nseg] / BM;
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&ctl->full[s], 1);
-      mbar_init(&ctl->empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&ctl->tfull[b], 1);
-      mbar_init(&ctl->tempty[b], 4);
-    }
-    mbar_init(&ctl->drain, 1);
-    mbar_init(&ctl->bgo[0], 1);
-    mbar_init(&ctl->bgo[1], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(&ctl->tmem_base)),
-                 "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-
-  const uint32_t tmem = ctl->tmem_base;
-  const int mt_total = ctl->mt_total;
-  const int ntn = p.ntiles_n;
-  const int tiles = mt_total * ntn;
-  volatile int* abort = &ctl->abort;
-
-  if (warp == 0) {
-    // Producer: one thread issues the TMA copies. An adapted tile's extra k-block takes the next
-    // stage after its K loop: the producer waits for that stage like any other and hands it to
-    // the builder warp (bgo), which fills it. Every waiter thus waits on every phase of its
-    // barriers in order, which a parity wait needs (it is ambiguous two phases away).
-    if (lane == 0 && int(blockIdx.x) < tiles) {
-      uint32_t it = 0, nl = 0;
-      for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x) {
-        int mt, nt;
-        tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-        const int row0 = mt * BM;
-        const int sg = seg_of_row(ctl, row0);
-        const CUtensorMap* mb = &p.tma_b[sg];
-        const int yb0 = EPI == EPI_SWIGLU ? nt * (NB / 2) : nt * NB;
-        const int yb1 = EPI == EPI_SWIGLU ? p.b_half + nt * (NB / 2) : nt * NB + NB / 2;
-        for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
-          const int s = int(it % STAGES);
-          if (!mbar_wait(&ctl->empty[s], ((it / STAGES) & 1u) ^ 1u, abort, p.err)) break;
-          const uint32_t sa = base + uint32_t(s) * STAGE_BYTES, sb = sa + A_BYTES;
-          mbar_expect_tx(&ctl->full[s], STAGE_BYTES);
-          tma_load_2d(sa, &p.tma_a, kb * BK, row0, &ctl->full[s]);
-          tma_load_2d(sb, mb, kb * BK, yb0, &ctl->full[s]);
-          tma_load_2d(sb + C::B_BYTES / 2, mb, kb * BK, yb1, &ctl->full[s]);
-        }
-        if constexpr (LR > 0) {
-          if (p.lblk[sg] != nullptr && !*abort) {  // the extra k-block's stage, for the builder
-            const int s = int(it % STAGES);
-            if (!mbar_wait(&ctl->empty[s], ((it / STAGES) & 1u) ^ 1u, abort, p.err)) break;
-            mbar_arrive(&ctl->bgo[nl & 1u]);
-            ++nl;
-            ++it;
-          }
-        }
-      }
-      // Stages still in flight: the last STAGES issued ones (all consumed unless aborting).
-      const uint32_t n_tail = it < STAGES ? it : STAGES;
-      for (uint32_t j = it - n_tail; j < it; ++j)
-        mbar_wait_drain(&ctl->full[j % STAGES], (j / STAGES) & 1u, p.err);
-    }
-  } else if (LR > 0 && warp == kBuilderWarp) {
-    // Builder (adapters only): walks the producer's tile sequence and counts its stages; for the
-    // n-th adapted tile it loads U and B' into registers when the tile starts, waits for the
-    // producer's n-th hand-off (bgo[n % 2]: at most two are outstanding, since the MMAs stop at
-    // the first unfilled stage and a tile has at least two TMA stages), writes the stage and
-    // marks it full. Lane 0 waits; the outcome is broadcast.
-    if (int(blockIdx.x) < tiles) {
-      uint32_t it = 0, nl = 0;
-      for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        int mt, nt;
-        tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-        const int sg = seg_of_row(ctl, mt * BM);
-        it += uint32_t(p.kblocks);
-        if (p.lblk[sg] == nullptr) continue;
-        LOps lops;
-        lops.load(p, p.lblk[sg], mt, nt, lane);
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait(&ctl->bgo[nl & 1u], (nl >> 1) & 1u, abort, p.err);
-        if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-        const int s = int(it % STAGES);
-        const uint32_t sa = base + uint32_t(s) * STAGE_BYTES, sb = sa + A_BYTES;
-        lops.store(smem_raw + (sa - raw), smem_raw + (sb - raw), lane);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // for the MMA reads
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&ctl->full[s]);
-        ++nl;
-        ++it;
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0 && int(blockIdx.x) < tiles) {
-      uint32_t it = 0, lt = 0;
-      for (int tile = blockIdx.x; tile < tiles && !*abort; tile += gridDim.x) {
-        bool lor = false;
-        if constexpr (LR > 0) {
-          int mt, nt;
-          tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-            lor = p.lblk[seg_of_row(ctl, mt * BM)] != nullptr;
-        }
-        const uint32_t b = lt & 1u;
-        if (!mbar_wait(&ctl->tempty[b], ((lt >> 1) & 1u) ^ 1u, abort, p.err)) break;
-        tc_fence_after();
-        const uint32_t dt = tmem + b * NB;
-        bool ok = true;
-        const int nkb = p.kblocks + (lor ? 1 : 0);
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = int(it % STAGES);
-          if (!mbar_wait(&ctl->full[s], (it / STAGES) & 1u, abort, p.err)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sa = base + uint32_t(s) * STAGE_BYTES, sb = sa + A_BYTES;
-          const uint64_t da = sw128_desc(sa), db = sw128_desc(sb);
-          if (LR == 0 || kb < p.kblocks) {
-#pragma unroll
-            for (int k = 0; k < BK / 16; ++k)  // +32 bytes along K per step inside the swizzle atom
-              tc_mma(dt, da + uint64_t(2 * k), db + uint64_t(2 * k), C::IDESC,
-                     (kb | k) != 0 ? 1u : 0u);
-          } else {  // the adapters' up projections: D += U B'^T over K' columns
-#pragma unroll
-            for (int k = 0; k < LOps::KL / 16; ++k)
-              tc_mma(dt, da + uint64_t(2 * k), db + uint64_t(2 * k), C::IDESC, 1u);
-          }
-          tc_commit(&ctl->empty[s]);
-        }
-        if (!ok) break;
-        tc_commit(&ctl->tfull[b]);
-        ++lt;
-      }
-      tc_commit(&ctl->drain);  // arrives once every MMA issued above has completed
-      mbar_wait_drain(&ctl->drain, 0, p.err);
-    }
-  } else if (warp >= 2 && warp < 6) {
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
-    uint32_t lt = 0;
-    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-      int mt, nt;
-      tile_coords(tile, mt_total, ntn, p.group_m, mt, nt);
-      const uint32_t b = lt & 1u;
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait(&ctl->tfull[b], (lt >> 1) & 1u, abort, p.err) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t taddr = tmem + b * NB + (uint32_t(q * 32) << 16);
-      // this warp's staging rows; row r of the warp's quarter goes to global row grow0 + r
-      uint8_t* stg = reinterpret_cast<uint8_t*>(ctl) + kCtlBytes + q * kOutWarpBytes;
-      const size_t grow0 = size_t(mt) * BM + q * 32;
-      store_tile<EPI, NB>(p, stg, taddr, grow0, nt, lane);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl->tempty[b]);
-      ++lt;
-    }
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(TMEM_COLS)
-                 : "memory");
-  }
-}
-
-// The expert GEMMs on CTA pairs: tiles of 256 rows x 256 columns, one MMA of M = 256 per K step
-// issued by the pair's leader over both CTAs' shared memory. Each CTA loads its 128 activation
-// rows and its half of the tile's 256 weight rows (GEMM13: rank 0 the W1 rows, rank 1 the W3
-// rows, i.e. the gate and up halves of N; GEMM2: 128 consecutive W2 rows each), so every weight
-// element is read from shared memory once for the rows of both CTAs: a third less shared-memory
-// traffic per MMA than the one-CTA tiles, and half the weight tiles fetched from L2 per tile row.
-// Roles as in gemm_tc_kernel, 6 stages of 32 KB:
-//   warp 0 (both CTAs) - TMA producer; the loads of both CTAs complete on the leader's full[s],
-//             on which the leader expects the pair's bytes; each CTA waits on its own empty[s];
-//   warp 1 - allocates the pair's TMEM (both CTAs); in the leader, issues the MMAs, whose commits
-//             arrive on empty[s] and tfull[b] of both CTAs;
-//   warps 2-5 (both CTAs) - epilogue of the CTA's 128 rows of the tile; they release the
-//             accumulator on the leader's tempty[b] (eight arrivals: four warps per CTA).
-// Segments are padded to 256 rows. Every wait is bounded. The leader drains its last stages'
-// copies (both CTAs' bytes), the peer waits (bounded) until its last stages were consumed, and
-// both CTAs leave through one cluster barrier after the leader's MMAs have completed, so neither
-// exits while the other may still read its shared memory or arrive on its barriers.
-constexpr int kPairRows = 2 * BM;
-constexpr int kPairStages = 6;
-constexpr int kPairStageBytes = A_BYTES + (BN / 2) * BK * 2;  // 128 activation + 128 weight rows
-constexpr int kPairTmemCols = 2 * BN;                          // two 128 x 256 accumulators
-constexpr uint32_t kPairIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(BN >> 3) << 17) |
-                                (uint32_t(kPairRows >> 4) << 24);
-constexpr int kPairSmem = kPairStages * kPairStageBytes + 1024 + kCtlBytes + 4 * kOutWarpBytes;
-static_assert(kPairSmem <= 227 * 1024, "shared memory");
-static_assert(kPairStages <= kMaxStages, "stage barriers");
-
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_tc_pair_kernel(const __grid_constant__ TcParams p) {
@@ -533,7 +217,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   volatile int* abort = &ctl->abort;
 
   if (warp == 0) {
-    if (lane == 0 && cid < tiles) {
+    if (cid < tiles && elect_one()) {
       uint32_t it = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
         int mt, nt;
@@ -562,7 +246,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    if (leader && lane == 0 && cid < tiles) {
+    if (leader && cid < tiles && elect_one()) {
       uint32_t it = 0, lt = 0;
       for (int tile = cid; tile < tiles && !*abort; tile += ncl) {
         const uint32_t b = lt & 1u;
@@ -638,7 +322,6 @@ bool encode_2d(CUtensorMap* m, const void* base, uint64_t cols, uint64_t rows) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-constexpr size_t kSmallSegGroupMB = 2;  // group budget when routed experts have few m-tiles
 // With CTA-pair tiles selected, layers whose routed experts average at least this many rows run
 // on pairs (segments padded to 256 rows); with fewer the extra padding would dominate.
 constexpr int kPairMinRows = 512;
@@ -647,18 +330,6 @@ int group_for(size_t a_tile_bytes, size_t budget_mb) {
   const size_t budget = budget_mb << 20;  // activation rows kept hot in L2 per group
   size_t g = budget / (a_tile_bytes ? a_tile_bytes : 1);
   return g < 1 ? 1 : int(g > 4096 ? 4096 : g);
-}
-
-template <int EPI, int LR>
-cudaError_t launch_one(const TcParams& p, int grid, cudaStream_t s) {
-  static cudaError_t attr = cudaFuncSetAttribute(
-      gemm_tc_kernel<EPI, LR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Tile::SMEM);
-  if (attr != cudaSuccess) return attr;
-  const int kid = EPI == EPI_SWIGLU ? kProfGemm13 : kProfGemm2;
-  prof_begin(kid, s);
-  gemm_tc_kernel<EPI, LR><<<grid, threads_for(LR), Tile::SMEM, s>>>(p);
-  prof_end(kid, s);
-  return cudaGetLastError();
 }
 
 // One pair per two SMs that can hold one at a time (one CTA per SM): a persistent grid of pairs
@@ -688,16 +359,6 @@ cudaError_t launch_pair(const TcParams& p, int num_sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int EPI>
-cudaError_t launch_rank(const TcParams& p, int rank, int num_sms, cudaStream_t s) {
-  switch (rank) {
-    case 0: return launch_one<EPI, 0>(p, num_sms, s);
-    case 8: return launch_one<EPI, 8>(p, num_sms, s);
-    case 16: return launch_one<EPI, 16>(p, num_sms, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
 }  // namespace
 
 bool tc_pair_tiles(int T, int K, int E, int lrank) {
@@ -706,8 +367,7 @@ bool tc_pair_tiles(int T, int K, int E, int lrank) {
 
 cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, int num_sms,
                           cudaStream_t s, int stages) {
-  const bool pair = pad == kPairRows;
-  if (pair ? a.lrank != 0 : pad != BM) return cudaErrorInvalidValue;
+  if (pad != kPairRows || a.lrank != 0) return cudaErrorInvalidValue;
   TcParams p13, p2;
   memset(&p13, 0, sizeof(p13));
   memset(&p2, 0, sizeof(p2));
@@ -735,40 +395,18 @@ cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, i
   p13.ntiles_n = int(w / (BN / 2));
   p13.ldo = int(w);
   p13.b_half = int(w);
-  // L2 budgets per group of m-tiles, from same-box sweeps over the Mixtral- and
-  // DeepSeek-V2-Lite-shaped T = 4096 layers: with several m-tiles per routed expert (Mixtral)
-  // GEMM13 is best at 24 MB and GEMM2 at 12 MB; with fewer than four on average (DeepSeek-V2-Lite:
-  // 64 experts) small groups of about one expert's rows win (GEMM13 0.55 -> 0.60 of peak)
-  // routed rows T * K: the permuted rows less the shared experts' and the segment padding
-  const size_t routed = size_t(mcap) - size_t(a.T) * (a.nseg - a.E) - size_t(a.nseg) * (pad - 1);
-  const bool small_segs = routed < size_t(4) * BM * a.E;
-  const size_t mb13 = small_segs ? kSmallSegGroupMB : 24, mb2 = small_segs ? kSmallSegGroupMB : 12;
-  p13.group_m = group_for(size_t(pad) * d * 2, mb13);
+  // L2 budgets per group of m-tiles, from sweeps over the Mixtral-shaped T = 4096 layer
+  p13.group_m = group_for(size_t(pad) * d * 2, 24);
   p2.out = a.o;
   p2.kblocks = int(w / BK);
   p2.ntiles_n = int(d / BN);
   p2.ldo = int(d);
   p2.b_half = 0;
-  p2.group_m = group_for(size_t(pad) * w * 2, mb2);
-  if (a.lrank > 0) {
-    const LoraOffsets lo = lora_offsets(a.d, a.w, a.lrank);
-    for (int sgi = 0; sgi < a.nseg; ++sgi) {
-      p13.lblk[sgi] = reinterpret_cast<const char*>(a.lblk[sgi]);
-      p2.lblk[sgi] = p13.lblk[sgi];
-    }
-    // U13 and U2 (bf16, from the down-projection launches) feed the extra k-blocks
-    p13.lug = reinterpret_cast<const uint16_t*>(a.u13);
-    p13.lb0 = lo.b1;
-    p13.lb1 = lo.b3;
-    p2.lug = reinterpret_cast<const uint16_t*>(a.u2);
-    p2.lb0 = lo.b2;
-  }
+  p2.group_m = group_for(size_t(pad) * w * 2, 12);
   cudaError_t e = cudaSuccess;
-  if (stages & 1)
-    e = pair ? launch_pair<EPI_SWIGLU>(p13, num_sms, s)
-             : launch_rank<EPI_SWIGLU>(p13, a.lrank, num_sms, s);
+  if (stages & 1) e = launch_pair<EPI_SWIGLU>(p13, num_sms, s);
   if (e != cudaSuccess || !(stages & 2)) return e;
-  return pair ? launch_pair<EPI_F32>(p2, num_sms, s) : launch_rank<EPI_F32>(p2, a.lrank, num_sms, s);
+  return launch_pair<EPI_F32>(p2, num_sms, s);
 }
 
 }  // namespace mcft

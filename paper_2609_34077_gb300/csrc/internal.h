@@ -271,8 +271,8 @@ cudaError_t launch_ffn_tile(const FfnArgs& a, int num_sms, cudaStream_t s, int s
 cudaError_t launch_ffn_decode(const FfnArgs& a, int num_sms, cudaStream_t s, int stages = 3,
                               int reserved = 0);  // bf16, T <= 64
 int decode_ksplit(int T);  // contraction split of the decode GEMM2 for T tokens
-// pad: rows per segment of the permutation, 128 (one-CTA tiles) or 256 (CTA-pair tiles, which
-// tc_pair_tiles chooses for layers without adapters whose routed experts average >= 512 rows).
+// pad: rows per segment of the permutation, 256: the CTA-pair tiles, which
+// tc_pair_tiles chooses, when selected, for layers without adapters whose routed experts average >= 512 rows).
 cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, int num_sms,
                           cudaStream_t s, int stages = 3);
 bool tc_pair_tiles(int T, int K, int E, int lrank);

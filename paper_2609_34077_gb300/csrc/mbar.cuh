@@ -1,5 +1,5 @@
-// Shared-memory mbarriers (sm_90+ PTX) with bounded waits, used by the tensor-core expert GEMMs
-// (gemm_tc.cu). Not part of the C ABI.
+// Shared-memory mbarriers (sm_90+ PTX) of the tensor-core expert GEMMs; their bounded waits are in
+// tc_ptx.cuh. Not part of the C ABI.
 #pragma once
 
 #include "common.cuh"
@@ -21,47 +21,4 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
                "r"(bytes)
                : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Wait for the phase of `parity` to complete; false if the kernel is aborting or 2 s passed.
-__device__ inline bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort,
-                                 unsigned* err) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t i = 1;; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 31) == 0) {
-      if (*abort) return false;
-      if (globaltimer_ns() - t0 > kTimeoutNs) {
-        *abort = 1;
-        set_error(err, kErrTimeout);
-        return false;
-      }
-    }
-  }
-}
-
-// Bounded wait used while draining (ignores the abort flag).
-__device__ inline void mbar_wait_drain(uint64_t* bar, uint32_t parity, unsigned* err) {
-  const uint64_t t0 = globaltimer_ns();
-  while (!mbar_try_wait(bar, parity)) {
-    if (globaltimer_ns() - t0 > kTimeoutNs) {
-      set_error(err, kErrTimeout);
-      return;
-    }
-  }
-}
-
 }  // namespace mcft
