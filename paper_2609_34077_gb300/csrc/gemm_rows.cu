@@ -26,14 +26,14 @@
 //   (1.57 PFLOP/s), GEMM2 184 -> 154 us (1.23): the MMAs and the power cap. The old tiles paid 12 % for
 //   padding and read 1.28 GB of DRAM where 0.69 GB does. Narrower token tiles and weights prefetched
 //   into L2 were slower.
-// * 200 tokens (19 rows an expert): HBM, the weights read once: GEMM13 145 -> 100 us, GEMM2 68 -> 56 us
-//   (525 and 264 MB of weights: 5.3 and 4.7 TB/s, the start and the last round of tiles included).
+// * 200 tokens (19 rows an expert): HBM, the weights read once: GEMM13 145 -> 97 us, GEMM2 68 -> 55 us
+//   (525 and 264 MB of weights: 5.4 and 4.8 TB/s, the start and the last round of tiles included).
 // * Mixtral shape, 4096 tokens (2048 rows an expert), GEMM13 1219 -> 1147 us, GEMM2 661 -> 637 us: the
 //   power cap.
 // The two threads that issue are what the loops wait for when they are not kept short: with the ring
 // walked under a lane test (operands moved to uniform registers one by one), tokens fetched as up to
 // four boxes and the peer's barrier address found per block, the rates above were GEMM13 300 and
-// GEMM2 175 us at 4096 DeepSeek tokens, 106 and 61 us at 200. One elected lane, one box per half tile
+// GEMM2 175 us at 4096 DeepSeek tokens, 106 and 61 us at 200 (six stages). One elected lane, one box per half tile
 // (hence a map for each size) and the addresses found once per tile gave the rest. Two k-blocks per
 // stage and per copy (5-D and 3-D boxes) were faster than the old loop and are slower than this one.
 // Eight epilogue warps rather than four, and a quotient without branches (silu_to_bf16): the SwiGLU of a
@@ -42,9 +42,14 @@
 //
 // Roles (both CTAs of a pair): warp 0 TMA producer (its 128 weight rows and its half of the tokens,
 // counted on the leader's full[s]); warp 1 allocates TMEM and, in the leader, issues the MMAs; warps
-// 2-9 read the CTA's 128 accumulator rows. A ring of 192 KB,
-// six stages of 32 KB with 256-token tiles and up to ten with narrower ones; two accumulators of 256
-// columns, so a tile's epilogue runs under the next tile's MMAs.
+// 2-9 read the CTA's 128 accumulator rows and store them from registers. Two accumulators of 256
+// columns, so a tile's epilogue runs under the next tile's MMAs. All of the shared memory is the ring,
+// 224 KB: the MMAs take a stage of a 256-token tile in 270 ns, so what the ring covers of a load's
+// latency is short. Seven stages of 32 KB there (and up to ten of narrower tiles; twelve were slower)
+// against six with a staging buffer for h beside them: 800 DeepSeek tokens 247 -> 239 us, 200 tokens
+// 166 -> 162, 4096 even (476 / 475). Stages of each tile's own size (more of them where the shared
+// experts' tiles are wide and the routed ones' narrow) cost the producer more than they gave: 200
+// tokens 171 us, 4096 498.
 //
 // With LoRA adapters (Section 3.2, Stage 2) an adapted tile appends p.nx k-blocks of one MMA each,
 // D += B' U^T: for GEMM13 B' is B1 on the gate rows (zeros on the up rows) with U = s A1 x, then B3 on
@@ -69,15 +74,11 @@ constexpr int kBoxes = 8;                     // token boxes of 16, 32, .. 128 r
 constexpr int kUBoxes = 4;                    // adapters' U: boxes of 16, 32, 64 and 128 rows, combined
 constexpr int kMaxStages = 10;
 constexpr int kABytes = 128 * BK * 2;         // a CTA's weight rows of a stage
-constexpr int kRingBytes = 6 * (kABytes + (kTileTok / 2) * BK * 2);
+constexpr int kRingBytes = 7 * (kABytes + (kTileTok / 2) * BK * 2);
 constexpr int kTmemCols = 2 * kTileTok;
 constexpr int kMaxExtra = 4;
 // instruction descriptor without N: D fp32, A and B bf16, both K-major, M = 256
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(256 >> 4) << 24);
-// GEMM13 output staging: 32 tokens x 64 bf16, two buffers per epilogue group; rows padded to 160
-// bytes, so the two rows a warp writes at once (32 bytes of each) fall into different banks
-constexpr int kStgRow = 160;
-constexpr int kStgBytes = 32 * kStgRow;
 
 enum { EPI_SWIGLU = 0, EPI_F32 = 1 };
 
@@ -109,7 +110,7 @@ struct Ctl {
   int first[kMaxSeg + 1];  // by position (segments in reverse order): first tile
 };
 constexpr int kCtlBytes = (int(sizeof(Ctl)) + 15) / 16 * 16;
-constexpr int kSmem = kRingBytes + 1024 + kCtlBytes + 2 * kEpiGroups * kStgBytes;
+constexpr int kSmem = kRingBytes + 1024 + kCtlBytes;
 static_assert(kSmem <= 227 * 1024, "shared memory");
 
 __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, int c0,
@@ -131,23 +132,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
         "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
         "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-}
-
-// Barrier of the four warps of an epilogue group, and the same with an AND over a flag (so that
-// either all of them leave the tile loop or none does: a warp alone at the barrier would wait for
-// ever).
-__device__ __forceinline__ void epi_sync(int grp) {
-  asm volatile("barrier.cta.sync %0, 128;" ::"r"(1 + grp) : "memory");
-}
-__device__ __forceinline__ int epi_all(int grp, int v) {
-  int r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.s32 q, %2, 0;\n barrier.cta.red.and.pred p, %1, 128, q;\n"
-      " selp.s32 %0, 1, 0, p;\n}"
-      : "=r"(r)
-      : "r"(1 + grp), "r"(v)
-      : "memory");
-  return r;
 }
 
 __device__ __forceinline__ int token_tiles(int rows) { return (rows + kTileTok - 1) / kTileTok; }
@@ -398,47 +382,37 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else {
     const int q = warp & 3, grp = (warp - 2) >> 2;  // TMEM lane quarter this warp may access; group
-    uint8_t* stg0 = reinterpret_cast<uint8_t*>(ctl) + kCtlBytes + grp * 2 * kStgBytes;
-    uint32_t lt = 0, chunk = 0;
+    uint32_t lt = 0;
     for (int tile = cid; tile < tiles; tile += ncl) {
       const TileAt t = tile_at(ctl, nseg, p.mtiles, p.group_x, tile);
       const uint32_t b = lt & 1u;
       int ok = 1;
       if (lane == 0) ok = mbar_wait_cl(&ctl->tfull[b], (lt >> 1) & 1u, abort, p.err) ? 1 : 0;
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!epi_all(grp, ok)) break;
+      if (!__shfl_sync(0xffffffffu, ok, 0)) break;
       tc_fence_after();
       const uint32_t taddr = tmem + b * kTileTok + (uint32_t(q * 32) << 16);
       // the groups take the 32-token chunks in turn
-      for (int c0 = grp * 32; c0 < t.n; c0 += 32 * kEpiGroups, ++chunk) {
+      for (int c0 = grp * 32; c0 < t.n; c0 += 32 * kEpiGroups) {
         uint32_t v[32];
         tmem_ld32(taddr + c0, v);
         tmem_ld_wait();
         if constexpr (EPI == EPI_SWIGLU) {
           // lanes 0-15 hold the gate and lanes 16-31 the up values of 16 outputs: lane pairs
-          // exchange, so that a low lane finishes the even columns and a high lane the odd ones
-          uint8_t* stg = stg0 + (chunk & 1u) * kStgBytes;
+          // exchange, so that a low lane finishes the even tokens and a high lane the odd ones, and
+          // a store writes one 32-byte sector of each of two rows
           const bool low = lane < 16;
-          uint16_t* dst = reinterpret_cast<uint16_t*>(stg + (low ? 0 : kStgRow)) + q * 16 + (lane & 15);
+          const int col = (t.mt * 2 + int(rank)) * 64 + q * 16 + (lane & 15);
+          const int m = t.n - c0 - (low ? 0 : 1);
+          uint16_t* dst = reinterpret_cast<uint16_t*>(p.out) +
+                          size_t(t.row0 + c0 + (low ? 0 : 1)) * p.ldo + col;
+          const bool in = col < p.ldo;
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
+          for (int i = 0; i < 16; ++i, dst += 2 * p.ldo) {
             const uint32_t mine = low ? v[2 * i] : v[2 * i + 1];
             const uint32_t got = __shfl_xor_sync(0xffffffffu, low ? v[2 * i + 1] : v[2 * i], 16);
             const float g = __uint_as_float(low ? mine : got), u = __uint_as_float(low ? got : mine);
-            dst[i * kStgRow] = f2bf(silu_to_bf16(g) * u);  // two staging rows (2 * kStgRow bytes) per i
-          }
-          epi_sync(grp);  // one per chunk: a buffer is written again two chunks later
-          const int col = (t.mt * 2 + int(rank)) * 64;
-          if (col < p.ldo) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const int r = q * 8 + i * 4 + (lane >> 3);
-              if (c0 + r < t.n) {
-                const uint4 w = *reinterpret_cast<const uint4*>(stg + r * kStgRow + (lane & 7) * 16);
-                *reinterpret_cast<uint4*>(reinterpret_cast<uint16_t*>(p.out) +
-                                          size_t(t.row0 + c0 + r) * p.ldo + col + (lane & 7) * 8) = w;
-              }
-            }
+            const uint16_t h = f2bf(silu_to_bf16(g) * u);
+            if (in && 2 * i < m) *dst = h;
           }
         } else {
           const int col = t.mt * 256 + int(rank) * 128 + q * 32 + lane;
