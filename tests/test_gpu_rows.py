@@ -69,6 +69,16 @@ def test_sizes_and_segments(d, w, T, first):
     _run(shape, T, _sized_ids(T, shape.K, shape.E, first), 200 + T)
 
 
+@pytest.mark.parametrize("d,w", [(64, 192), (960, 704)])
+@pytest.mark.parametrize("rank", [0, 8])
+def test_every_token_box(d, w, rank):
+    """Segments whose tiles are 32, 64, .. 256 tokens wide in one launch: each of the eight boxes a half
+    tile is fetched as, the last rows of a box belonging to the next segment, or past the end."""
+    shape = _shape(d, w, E=12)
+    first = [1, 40, 70, 100, 130, 165, 200, 230]
+    _run(shape, 600, _sized_ids(600, 2, 12, first), 240, rank)
+
+
 @pytest.mark.parametrize("d,w", [(64, 64), (320, 192), (512, 256)])
 @pytest.mark.parametrize("rank", [8, 16])
 def test_adapters(d, w, rank):
