@@ -7,12 +7,13 @@
 // and the 32 up values of the same outputs, joined in registers): 32 contraction elements per step,
 // copied to shared memory three steps ahead (cp.async, rows padded by 16 bytes), 4 tokens x 8 (GEMM13)
 // or 4 (GEMM2) values per thread, so 12 (8) 16-byte shared loads feed 128 (64) multiply-adds.
-// 8 products are summed first, 4 such sums make a step's, and the steps' are added to the total: one
-// running sum's error grows with the square root of its length, and the row-wise kernels add 32 lanes'
-// short sums in a tree. Error of y against 64 bits at d = 256, w = 512: 1.8e-7, row-wise 1.7e-7 (with
-// 32 products in one sum 2.2e-7).
+// 8 products are summed first, 4 such sums make a step's, and what adding a step to the total drops is
+// carried into the next step (compensated summation): one running sum's error grows with the square root
+// of its length, and the row-wise kernels add 32 lanes' short sums in a tree. Error of a dot product of
+// normal values against 64 bits: 7.4e-8 at every length, row-wise 8.1e-8 at 256 and 1.2e-7 at 1024
+// elements (8.8e-8 and 1.3e-7 with the steps simply added, 6 % faster).
 // Measured (GB300, d = 256, w = 512, 8 experts, 512 tokens on 4 of them, events around each launch):
-// GEMM13 33 us and GEMM2 27 us against 168 and 179 us row-wise; the multiply-adds alone take 11 us at
+// GEMM13 35 us and GEMM2 29 us against 168 and 179 us row-wise; the multiply-adds alone take 11 us at
 // the fp32 rate: the tile counts (256 and 128) leave the SMs few warps to hide shared loads behind.
 // Warps take 16 tokens each, and one without tokens skips its arithmetic.
 #include "common.cuh"
@@ -148,11 +149,11 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_tile_kernel(const __grid_cons
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[4][NC];  // [token][weight row]
+    float acc[4][NC], sum[4][NC];  // [token][weight row]: total, and the step's with what it lost
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < NC; ++j) acc[i][j] = 0.f;
+      for (int j = 0; j < NC; ++j) acc[i][j] = sum[i][j] = 0.f;
     const bool busy = warp * 16 < n;
     __syncthreads();  // the previous item's steps are read
     for (int st = 0; st < kDepth - 1; ++st) copy(st);
@@ -163,7 +164,6 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_tile_kernel(const __grid_cons
       if (busy) {
         const float* xa = smem + (st % kDepth) * kStep + t0 * kPitch;
         const float* wb = smem + (st % kDepth) * kStep + (TM + c0) * kPitch;
-        float sum[4][NC];
 #pragma unroll
         for (int k8 = 0; k8 < BK; k8 += 8) {
           float part[4][NC];
@@ -187,12 +187,17 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_tile_kernel(const __grid_cons
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < NC; ++j) sum[i][j] = k8 == 0 ? part[i][j] : sum[i][j] + part[i][j];
+            for (int j = 0; j < NC; ++j) sum[i][j] += part[i][j];
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < NC; ++j) acc[i][j] += sum[i][j];
+          for (int j = 0; j < NC; ++j) {
+            // what the addition drops stays in sum, for the next step (nothing beside an infinite total)
+            const float t = acc[i][j] + sum[i][j], lost = sum[i][j] - (t - acc[i][j]);
+            sum[i][j] = fabsf(t) < INFINITY ? lost : 0.f;
+            acc[i][j] = t;
+          }
       }
     }
     const void* lblk = a.lrank ? a.lblk[s] : nullptr;
@@ -205,9 +210,9 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_tile_kernel(const __grid_cons
 #pragma unroll
       for (int j = 0; j < TN / 8; ++j) {
         const int row = r0 + c0 + 8 * j;
-        float g = acc[i][j];
+        float g = acc[i][j] + sum[i][j];
         if constexpr (STAGE == 13) {
-          float u = acc[i][j + TN / 8];
+          float u = acc[i][j + TN / 8] + sum[i][j + TN / 8];
           if (lblk) {  // LoRA: + s B1 (A1 x), + s B3 (A3 x)
             const LoraOffsets lo = lora_offsets(a.d, a.w, a.lrank);
             const float* m = a.u13 + size_t(q) * 2 * a.lrank;

@@ -40,6 +40,22 @@ def test_tiles_against_the_oracle(d, w, S, T, first):
     check_output(y, oracle.ffn.moe_layer(*ref), TOL_F32, shape.name)
 
 
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3e38])
+@pytest.mark.parametrize("k", [0, 40, 255])
+def test_infinities_as_on_the_row_path(value, k):
+    """An infinite, undefined or overflowing input in any step of the contraction: the token's outputs are
+    infinite and undefined where the row-wise kernels' (a batch of one token) are; other tokens finite."""
+    shape, T = _shape(256, 128), 70
+    ids = _sized_ids(T, 2, 4, [17, 64])
+    dev, _ = _args(shape, T, ids, 330)
+    dev[1][3, k] = value
+    y = M.mcft_moe_forward(*dev)
+    y1 = M.mcft_moe_forward(dev[0], *(v[3:4].contiguous() for v in dev[1:4]), *dev[4:])
+    M.mcft_device_error()
+    assert torch.equal(torch.isnan(y[3:4]), torch.isnan(y1)) and torch.equal(torch.isinf(y[3:4]), torch.isinf(y1))
+    assert torch.isfinite(torch.cat([y[:3], y[4:]])).all()
+
+
 @pytest.mark.parametrize("rank", [8, 16])
 def test_tiles_with_adapters(rank):
     shape, T, seed = _shape(128, 192, S=1), 90, 310
