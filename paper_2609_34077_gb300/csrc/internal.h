@@ -167,7 +167,7 @@ struct FfnArgs {
   void* h;                       // [mcap, w] fp32 (rowwise) or bf16 (tensor cores, decode)
   float* o;                      // [ksplit][mcap, d] fp32
   size_t o_plane;                // elements between partial planes of o
-  int T, K, d, w, nseg, E, ksplit;
+  int T, d, w, nseg, E, ksplit;
   unsigned* err;
   // Expert addresses written on the device by a cache step (NULL: use wblk), that step's hit
   // mask, and which segments this launch computes: 0 all, 1 hit experts and shared experts,
@@ -208,6 +208,9 @@ struct FfnArgs {
   const unsigned long long* fsrc;
   size_t fbytes;
   int nfetch;
+  // For the host's choice of item sizes. Last: among the first integers it moved the others' offsets, and
+  // the decode build of 17 to 64 tokens, which takes all 128 registers, spilled.
+  int K;
 };
 
 // Bytes per work unit of the device-driven fetch: the granule of its landed stamps.
