@@ -78,27 +78,13 @@ unsigned long long test_wait_limit_ns() {
 
 bool test_withhold_gemm13() { return g_inject_withhold.load() != 0; }
 
-namespace {
-
-constexpr int kMaxDevices = 64;
-
-int current_device() {
-  int dev = 0;
-  cudaGetDevice(&dev);
-  return dev;
-}
-
-}  // namespace
-
 int num_sms() {
-  static int cache[kMaxDevices] = {0};
-  const int dev = current_device();
-  if (dev < kMaxDevices && cache[dev]) return cache[dev];
-  int n = 0;
-  cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-  if (n <= 0) n = 1;
-  if (dev < kMaxDevices) cache[dev] = n;
-  return n;
+  static PerDeviceInt sms;
+  return sms.get([] {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, current_device());
+    return n > 0 ? n : 1;
+  });
 }
 
 namespace {

@@ -233,13 +233,12 @@ __global__ void __launch_bounds__(kThreads, 3) ffn_tile_kernel(const __grid_cons
 
 template <int STAGE>
 cudaError_t launch_stage(const FfnArgs& a, int num_sms, cudaStream_t s) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      ffn_tile_kernel<STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes<STAGE>);
-  if (attr != cudaSuccess) return attr;
+  static SmemOptIn smem;
+  cudaError_t e = smem.allow(reinterpret_cast<const void*>(ffn_tile_kernel<STAGE>), kSmemBytes<STAGE>);
+  if (e != cudaSuccess) return e;
   const int kid = STAGE == 13 ? kProfFfn13 : kProfFfn2;
   prof_begin(kid, s);
-  const cudaError_t e = launch_pdl(ffn_tile_kernel<STAGE>, dim3(3 * num_sms), dim3(kThreads),
-                                   kSmemBytes<STAGE>, s, a);
+  e = launch_pdl(ffn_tile_kernel<STAGE>, dim3(3 * num_sms), dim3(kThreads), kSmemBytes<STAGE>, s, a);
   prof_end(kid, s);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -477,27 +477,16 @@ bool encode_gate_up(CUtensorMap* m, const void* base, uint64_t cols, uint64_t ro
 
 template <int EPI, typename P>
 cudaError_t launch_rows(const P& p, int num_sms, cudaStream_t s) {
-  static cudaError_t attr = cudaFuncSetAttribute(
-      gemm_rows_kernel<EPI, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  if (attr != cudaSuccess) return attr;
-  // a persistent grid of pairs that all run at once
-  static const int pairs = [num_sms] {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(num_sms & ~1));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmem;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_rows_kernel<EPI, P>, &cfg) != cudaSuccess) {
-      (void)cudaGetLastError();
-      n = 0;
-    }
-    return n;
-  }();
+  static SmemOptIn smem;
+  static ResidentClusters resident;  // a persistent grid of pairs that all run at once
+  const void* fn = reinterpret_cast<const void*>(gemm_rows_kernel<EPI, P>);
+  cudaError_t e = smem.allow(fn, kSmem);
+  if (e != cudaSuccess) return e;
+  const int pairs = resident.get(fn, num_sms & ~1, kThreads, kSmem);
   if (pairs < 1) return cudaErrorInvalidConfiguration;
   const int kid = EPI == EPI_SWIGLU ? kProfGemm13 : kProfGemm2;
   prof_begin(kid, s);
-  const cudaError_t e =
-      launch_pdl(gemm_rows_kernel<EPI, P>, dim3(2 * pairs), dim3(kThreads), kSmem, s, p);
+  e = launch_pdl(gemm_rows_kernel<EPI, P>, dim3(2 * pairs), dim3(kThreads), kSmem, s, p);
   prof_end(kid, s);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

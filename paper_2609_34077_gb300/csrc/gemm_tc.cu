@@ -336,21 +336,12 @@ int group_for(size_t a_tile_bytes, size_t budget_mb) {
 // that all run at once, so no pair's tiles wait for another pair to exit.
 template <int EPI>
 cudaError_t launch_pair(const TcParams& p, int num_sms, cudaStream_t s) {
-  static cudaError_t attr = cudaFuncSetAttribute(
-      gemm_tc_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
-  if (attr != cudaSuccess) return attr;
-  static const int pairs = [num_sms] {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(num_sms & ~1));
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kPairSmem;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, gemm_tc_pair_kernel<EPI>, &cfg) != cudaSuccess) {
-      (void)cudaGetLastError();
-      n = 0;
-    }
-    return n;
-  }();
+  static SmemOptIn smem;
+  static ResidentClusters resident;
+  const void* fn = reinterpret_cast<const void*>(gemm_tc_pair_kernel<EPI>);
+  const cudaError_t e = smem.allow(fn, kPairSmem);
+  if (e != cudaSuccess) return e;
+  const int pairs = resident.get(fn, num_sms & ~1, kThreads, kPairSmem);
   if (pairs < 1) return cudaErrorInvalidConfiguration;
   const int kid = EPI == EPI_SWIGLU ? kProfGemm13Pair : kProfGemm2Pair;
   prof_begin(kid, s);

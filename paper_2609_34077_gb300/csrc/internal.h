@@ -11,6 +11,7 @@
 
 #include "../../include/mcft.h"
 #include "common.cuh"
+#include "per_device.h"
 
 namespace mcft {
 

@@ -411,10 +411,10 @@ cudaError_t launch_route_tile_t(const RouteArgs& a, cudaStream_t s) {
   constexpr int stage = route_tile_stage(TT, NTW), partial = 2 * 64 * (NTW * 8 + 1) * 4;
   constexpr int most = kTileRingBytes / stage < kTileMaxStages ? kTileRingBytes / stage : kTileMaxStages;
   static_assert(most >= 2, "the ring needs two stages");
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(route_tile_cluster_kernel<NTW, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           most * stage > partial ? most * stage : partial);
-  if (attr != cudaSuccess) return attr;
+  static SmemOptIn optin;
+  const cudaError_t e = optin.allow(reinterpret_cast<const void*>(route_tile_cluster_kernel<NTW, TT>),
+                                    most * stage > partial ? most * stage : partial);
+  if (e != cudaSuccess) return e;
   // a slice shorter than the ring takes one stage more than it has: all of it is copied at once
   const int units = (a.d / 64 + kTileCluster - 1) / kTileCluster;
   const int depth = max(2, min(most, (units * 64 + kTileK - 1) / kTileK + 1));
