@@ -36,7 +36,7 @@
 // GEMM2 175 us at 4096 DeepSeek tokens, 106 and 61 us at 200 (six stages). One elected lane, one box per half tile
 // (hence a map for each size) and the addresses found once per tile gave the rest. Two k-blocks per
 // stage and per copy (5-D and 3-D boxes) were faster than the old loop and are slower than this one.
-// Eight epilogue warps rather than four, and a quotient without branches (silu_to_bf16): the SwiGLU of a
+// Eight epilogue warps rather than four, and a quotient without branches (silu_branchless): the SwiGLU of a
 // tile took about 28,000 cycles on four warps, more than the MMAs of a 2048-long contraction (16,400).
 // d = 960, w = 704 (15 k-blocks), 16 experts: GEMM13 at T = 4096 99 -> 63 us by the quotient alone.
 //
@@ -406,13 +406,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           uint16_t* dst = reinterpret_cast<uint16_t*>(p.out) +
                           size_t(t.row0 + c0 + (low ? 0 : 1)) * p.ldo + col;
           const bool in = col < p.ldo;
+          bool regular = true;
 #pragma unroll
-          for (int i = 0; i < 16; ++i, dst += 2 * p.ldo) {
+          for (int i = 0; i < 16; ++i) {
             const uint32_t mine = low ? v[2 * i] : v[2 * i + 1];
             const uint32_t got = __shfl_xor_sync(0xffffffffu, low ? v[2 * i + 1] : v[2 * i], 16);
-            const float g = __uint_as_float(low ? mine : got), u = __uint_as_float(low ? got : mine);
-            const uint16_t h = f2bf(silu_to_bf16(g) * u);
-            if (in && 2 * i < m) *dst = h;
+            v[2 * i] = low ? mine : got;
+            v[2 * i + 1] = low ? got : mine;
+            const float g = __uint_as_float(v[2 * i]);
+            regular &= silu_regular(g);
+            const uint16_t h = f2bf(silu_branchless(g) * __uint_as_float(v[2 * i + 1]));
+            if (in && 2 * i < m) dst[2 * i * size_t(p.ldo)] = h;
+          }
+          if (!regular) {  // rare: this lane's values again, by IEEE division
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (in && 2 * i < m)
+                dst[2 * i * size_t(p.ldo)] = f2bf(silu(__uint_as_float(v[2 * i])) * __uint_as_float(v[2 * i + 1]));
           }
         } else {
           const int col = t.mt * 256 + int(rank) * 128 + q * 32 + lane;

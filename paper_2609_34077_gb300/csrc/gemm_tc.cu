@@ -114,10 +114,19 @@ __device__ __forceinline__ void store_tile(const TcParams& p, uint8_t* stg, uint
         tmem_ld16(taddr + NB / 2 + c0 + c, u);
         tmem_ld_wait();
         uint32_t pk[8];
+        bool regular = true;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          pk[i] = pack2bf(silu_to_bf16(__uint_as_float(g[2 * i])) * __uint_as_float(u[2 * i]),
-                          silu_to_bf16(__uint_as_float(g[2 * i + 1])) * __uint_as_float(u[2 * i + 1]));
+        for (int i = 0; i < 8; ++i) {
+          regular &= silu_regular(__uint_as_float(g[2 * i])) && silu_regular(__uint_as_float(g[2 * i + 1]));
+          pk[i] = pack2bf(silu_branchless(__uint_as_float(g[2 * i])) * __uint_as_float(u[2 * i]),
+                          silu_branchless(__uint_as_float(g[2 * i + 1])) * __uint_as_float(u[2 * i + 1]));
+        }
+        if (!regular) {  // rare: this lane's values again, by IEEE division
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            pk[i] = pack2bf(silu(__uint_as_float(g[2 * i])) * __uint_as_float(u[2 * i]),
+                            silu(__uint_as_float(g[2 * i + 1])) * __uint_as_float(u[2 * i + 1]));
+        }
         uint4* sw = reinterpret_cast<uint4*>(stg + lane * kOutRowBytes + c * 2);
         sw[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         sw[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
