@@ -128,11 +128,11 @@ unsigned* device_error_word() {
   return static_cast<unsigned*>(p);
 }
 
-WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank, bool no_tc) {
+WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank, bool compact) {
   WsLayout L{};
   L.lrank = lrank;
   const bool aligned = tc_aligned(d, w);
-  L.tc = dtype == MCFT_BF16 && T > 64 && !no_tc;
+  L.tc = dtype == MCFT_BF16 && T > 64;
   L.decode = !L.tc && dtype == MCFT_BF16;
   L.ks = L.decode ? decode_ksplit(T) : 1;
   const bool pair = L.tc && aligned && g_tc_tiles.load() == MCFT_TC_TILES_CTA_PAIR &&
@@ -154,8 +154,9 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   L.pos = o;  o = align256(o + sizeof(int) * size_t(T) * K);
   L.perm = o; o = align256(o + sizeof(int) * size_t(L.mcap));
   L.done = o; o = align256(o + sizeof(int) * (nseg + kClaimSlots));
-  L.xp = o;   o = align256(o + (L.tc ? size_t(L.mcap) * d * 2 : 0));
+  L.xp = o;   o = align256(o + (L.tc && !compact ? size_t(L.mcap) * d * 2 : 0));
   L.h = o;    o = align256(o + size_t(L.mcap) * w * (dtype == MCFT_BF16 ? 2 : 4));
+  if (compact) L.xp = o;
   L.o = o;    o = align256(o + size_t(L.ks) * L.mcap * d * 4);
   L.u13 = o;  o = align256(o + size_t(L.mcap) * 2 * lrank * 4);
   L.u2 = o;   o = align256(o + size_t(L.mcap) * lrank * 4);
@@ -397,7 +398,7 @@ struct LoraArgs {
 mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, const int32_t* idx,
                          const float* gate, const void* const* experts, const void* const* shared,
                          const LoraArgs* lora, void* y, void* workspace, size_t ws_bytes,
-                         cudaStream_t stream, bool no_tc = false) {
+                         cudaStream_t stream, bool compact = false) {
   mcft_status st = check_desc(desc);
   if (st != MCFT_OK) return st;
   if (T < 0) return fail(MCFT_ERR_INVALID, "T = %d < 0", T);
@@ -411,7 +412,7 @@ mcft_status forward_impl(const mcft_layer_desc* desc, const void* x, int T, cons
     return fail(MCFT_ERR_INVALID, "x and y must be 16-byte aligned");
   const int E = desc->E, S = desc->n_shared, K = desc->K;
   const int lrank = lora ? lora->rank : 0;
-  const WsLayout L = ws_layout(desc->d, E, K, desc->w, S, desc->dtype, T, lrank, no_tc);
+  const WsLayout L = ws_layout(desc->d, E, K, desc->w, S, desc->dtype, T, lrank, compact);
   if (ws_bytes < L.total)
     return fail(MCFT_ERR_INVALID, "workspace of %zu bytes < %zu needed", ws_bytes, L.total);
   for (int e = 0; e < E; ++e)
@@ -927,10 +928,9 @@ mcft_status mcft_moe_forward_cached(const mcft_layer_desc* desc, const void* x, 
 
 namespace mcft {
 
-mcft_status forward_decode_layout(const mcft_layer_desc* desc, const void* x, int T,
-                                  const int32_t* idx, const float* gate, const void* const* experts,
-                                  const void* const* shared, void* y, void* workspace,
-                                  size_t ws_bytes, cudaStream_t stream) {
+mcft_status forward_compact(const mcft_layer_desc* desc, const void* x, int T, const int32_t* idx,
+                            const float* gate, const void* const* experts, const void* const* shared,
+                            void* y, void* workspace, size_t ws_bytes, cudaStream_t stream) {
   return forward_impl(desc, x, T, idx, gate, experts, shared, nullptr, y, workspace, ws_bytes, stream,
                       true);
 }

@@ -87,9 +87,9 @@ struct WsLayout {
   int ks;         // partial planes of o (contraction split of the decode GEMM2)
   size_t hdr, cnt, off, pos, perm, done, xp, h, o, u13, u2, total;
 };
-// no_tc: the layout of the decode kernels whatever T is.
+// compact: xp takes o's memory (GEMM13 has read the permuted activations when GEMM2, which writes o, starts).
 WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0,
-                   bool no_tc = false);
+                   bool compact = false);
 // Layer sizes that fill the 128 x 256 tiles of gemm_tc.cu.
 inline bool tc_aligned(int d, int w) { return d % 256 == 0 && w % 128 == 0; }
 
@@ -435,11 +435,10 @@ cudaError_t launch_mask_grad(const MaskGradArgs& a, cudaStream_t s);
 unsigned* device_error_word();  // device address of the current device's error word
 mcft_status set_error_message(mcft_status st, const char* msg);  // mcft_last_error() text
 
-// mcft_moe_forward on the decode kernels and their workspace layout whatever T is (any d and w).
-mcft_status forward_decode_layout(const mcft_layer_desc* desc, const void* x, int T,
-                                  const int32_t* idx, const float* gate, const void* const* experts,
-                                  const void* const* shared, void* y, void* workspace,
-                                  size_t ws_bytes, cudaStream_t stream);
+// mcft_moe_forward on the compact workspace layout.
+mcft_status forward_compact(const mcft_layer_desc* desc, const void* x, int T, const int32_t* idx,
+                            const float* gate, const void* const* experts, const void* const* shared,
+                            void* y, void* workspace, size_t ws_bytes, cudaStream_t stream);
 
 // The device-driven cached forward (mcft_moe_forward_cached); permuted = the workspace already
 // holds this call's permutation (written by the fused prologue), so it is not recomputed.

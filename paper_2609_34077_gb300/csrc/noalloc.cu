@@ -73,11 +73,17 @@ extern "C" mcft_status mcft_moe_forward_noalloc(const mcft_layer_desc* desc, con
   size_t need = 0;
   mcft_status st = mcft_moe_workspace_size(desc, T, &need);
   if (st != MCFT_OK) return st;
-  // sizes off the 128 x 256 tiles also run on the decode kernels, whose layout is smaller
-  const bool compact =
-      need > kScratchBytes && desc->dtype == MCFT_BF16 && !tc_aligned(desc->d, desc->w);
-  if (compact)
-    need = ws_layout(desc->d, desc->E, desc->K, desc->w, desc->n_shared, desc->dtype, T, 0, true).total;
+  // d % 256 != 0 or w % 128 != 0: the array serves the batches that it served before these sizes had a
+  // section for the permuted activations
+  const bool compact = need > kScratchBytes && desc->dtype == MCFT_BF16 && T > 64 &&
+                       !tc_aligned(desc->d, desc->w);
+  if (compact) {
+    st = mcft_moe_workspace_size(desc, 64, &need);
+    if (st != MCFT_OK) return st;
+    const size_t total =
+        ws_layout(desc->d, desc->E, desc->K, desc->w, desc->n_shared, desc->dtype, T, 0, true).total;
+    need = need > total ? need : total;
+  }
   if (need > kScratchBytes) {
     char msg[256];
     snprintf(msg, sizeof(msg),
@@ -90,6 +96,6 @@ extern "C" mcft_status mcft_moe_forward_noalloc(const mcft_layer_desc* desc, con
   st = scratch_address(&scratch);
   if (st != MCFT_OK) return st;
   if (compact)
-    return forward_decode_layout(desc, x, T, idx, gate, experts, shared, y, scratch, kScratchBytes, stream);
+    return forward_compact(desc, x, T, idx, gate, experts, shared, y, scratch, kScratchBytes, stream);
   return mcft_moe_forward(desc, x, T, idx, gate, experts, shared, y, scratch, kScratchBytes, stream);
 }
