@@ -307,13 +307,15 @@ mcft_status mcft_mask_grad(const mcft_layer_desc* desc, const int32_t* idx, cons
  *    permutation and the FFN of the hits run on compute_stream; then compute_stream waits for the
  *    copies and computes the fetched experts.
  * Then the combine. Results equal mcft_moe_forward's with the same experts, bit for bit (a decode
- * work item has the same shape and summation order whichever launch computes its expert).
+ * work item, and a tile of the tensor-core GEMMs, has the same shape and summation order whichever
+ * launch computes its expert).
  * Section 3.1 Eq. topk (the layer); Section 1 and Section 3.1 "Preliminaries" (every miss is a fetch
  * from host memory).
  *   cache  created with host blocks (not accounting-only); its E and expert size match desc
  *   other arguments as for mcft_moe_forward (the routed expert addresses come from the cache)
- * Supports the decode path (bf16 with T <= 64, or fp32); larger bf16 calls return
- * MCFT_ERR_UNSUPPORTED (use mcft_fetch_experts + mcft_moe_forward). Asynchronous. */
+ * Supports fp32, bf16 with T <= 64, and bf16 of any T where d % 256 != 0 or w % 128 != 0; larger
+ * bf16 calls of the other sizes return MCFT_ERR_UNSUPPORTED (use mcft_fetch_experts +
+ * mcft_moe_forward). Asynchronous. */
 mcft_status mcft_moe_forward_cached(const mcft_layer_desc* desc, const void* x, int T,
                                     const int32_t* idx, const float* gate, mcft_cache* cache,
                                     int layer, const void* const* shared, void* y, void* workspace,

@@ -1056,10 +1056,18 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
   // 2. meanwhile: permutation (unless the fused prologue wrote it into this workspace) and the
   //    experts that were hits (and the shared experts)
   if (!permuted) {
-    PermuteArgs pa{idx, T, K, E, S, L.pad, L.mcap, hdr, cnt, off, pos, perm, err, done};
+    PermuteArgs pa{idx, T, K, E, S, L.pad, L.mcap, hdr, cnt, off, pos, perm, err, done, L.tc ? 1 : 0};
     e = launch_permute(pa, compute_stream);
     if (e != cudaSuccess) return cuda_fail(e, "permute kernel launch");
   }
+  if (L.tc) {
+    SpreadArgs sa{x, pos, perm, off, cnt, hdr, ws + L.xp, T, desc->d, K, E, S, L.pad};
+    e = launch_spread(sa, compute_stream);
+    if (e != cudaSuccess) return cuda_fail(e, "spread kernel launch");
+  }
+  const CacheBlocks blocks{{c->d_slots + size_t(layer) * c->B * c->expert_bytes, c->d_staging},
+                           {c->B, c->n_staging},
+                           c->expert_bytes};
   FfnArgs fa{};
   fa.x = x;
   fa.off = off;
@@ -1087,8 +1095,9 @@ mcft_status forward_cached_impl(const mcft_layer_desc* desc, const void* x, int 
     fa.phase = phase;
     if (phase == 2) MCFT_CUDA(cudaStreamWaitEvent(compute_stream, c->ev_copy, 0));
     const int reserved = phase == 1 || queued > 0 ? fetch_blocks() : 0;
-    e = desc->dtype == MCFT_BF16 ? launch_ffn_decode(fa, num_sms(), compute_stream, 3, reserved)
-                 : launch_ffn_rowwise(fa, desc->dtype, num_sms(), compute_stream);
+    e = L.rows     ? launch_ffn_rows_cached(fa, blocks, ws + L.xp, L.mcap, num_sms(), compute_stream)
+        : L.decode ? launch_ffn_decode(fa, num_sms(), compute_stream, 3, reserved)
+                   : launch_ffn_rowwise(fa, desc->dtype, num_sms(), compute_stream);
     if (e != cudaSuccess) return cuda_fail(e, "expert FFN launch");
   }
   CombineArgs ca{fa.o, gate, pos, off, hdr, y, T, desc->d, K, E, S, L.ks, fa.o_plane};

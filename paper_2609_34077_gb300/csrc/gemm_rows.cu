@@ -57,8 +57,13 @@
 // B' = B2, U = s A2 h. The zeros are TMA out-of-bounds fill: the adapter matrices are r columns wide
 // under boxes of 64, and the W1 / W3 dimension of the box is one plane long, entered at 0 or at -1.
 //
+// A cached forward's launch (RowsCacheParams) finds its weights in the cache step's device table. The other
+// launches carry none of that code. Per tile everything is as in the plain launch, hence the same bits.
+//
 // Every wait is bounded: after 2 s the kernel records MCFT_ERR_TIMEOUT, stops issuing, waits (bounded)
 // for its copies and MMAs in flight, frees TMEM and returns.
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 #include "tc_ptx.cuh"
@@ -100,7 +105,19 @@ struct RowsLoraParams : RowsParams {
   int nx;
 };
 
-static_assert(sizeof(RowsLoraParams) <= 32764, "kernel parameters");
+// A cached forward: the routed experts' blocks are in the layer's cache slots or in the staging buffers,
+// where the device table of the cache step says; their maps cover all blocks of either kind, with the block
+// as the last coordinate. One launch computes the segments of one phase (seg_in_phase).
+struct RowsCacheParams : RowsParams {
+  CUtensorMap blocks[2];  // slots, staging buffers
+  const unsigned long long* wtab;   // [E] block addresses
+  const unsigned long long* ready;  // hit mask
+  unsigned long long base[2], bytes;
+  int count[2];
+  int phase;
+};
+
+static_assert(sizeof(RowsLoraParams) <= 32764 && sizeof(RowsCacheParams) <= 32764, "kernel parameters");
 
 struct Ctl {
   uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
@@ -108,7 +125,9 @@ struct Ctl {
   int abort, tiles, stages, stage_bytes;
   int off[kMaxSeg + 1];
   int first[kMaxSeg + 1];  // by position (segments in reverse order): first tile
+  int block[kMaxE];        // cached forward: block of each routed expert, staging buffers from kStaging
 };
+constexpr int kStaging = 1 << 24;  // (more blocks than a GPU can hold)
 constexpr int kCtlBytes = (int(sizeof(Ctl)) + 15) / 16 * 16;
 constexpr int kSmem = kRingBytes + 1024 + kCtlBytes;
 static_assert(kSmem <= 227 * 1024, "shared memory");
@@ -119,6 +138,24 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap
       "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar_cluster)
+      : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* map, int c0,
+                                                 int c1, int c2, uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar_cluster)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1,
+                                                 int c2, int c3, int c4, uint32_t bar_cluster) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4),
+      "r"(bar_cluster)
       : "memory");
 }
 
@@ -174,10 +211,17 @@ __device__ __forceinline__ TileAt tile_at(const Ctl* c, int nseg, int mtiles, in
 
 __device__ __forceinline__ bool in_mask(const uint32_t* m, int s) { return (m[s >> 5] >> (s & 31)) & 1u; }
 
+// The segments of a cached forward's launch: hits and shared experts (phase 1), the others (phase 2).
+__device__ __forceinline__ bool rows_in_phase(const RowsCacheParams& p, int s) {
+  const bool hit = s >= p.E || ((*p.ready >> s) & 1ull);
+  return p.phase == 1 ? hit : !hit;
+}
+
 template <int EPI, typename P>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     gemm_rows_kernel(const __grid_constant__ P p) {
-  constexpr bool LORA = sizeof(P) == sizeof(RowsLoraParams);
+  constexpr bool LORA = std::is_same_v<P, RowsLoraParams>;
+  constexpr bool CACHED = std::is_same_v<P, RowsCacheParams>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;  // the same offsets in both CTAs
@@ -217,14 +261,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const int s = lane + 32 * j;
       if (s <= nseg) ctl->off[s] = p.off[s];
     }
+    if constexpr (CACHED) {
+      for (int e = lane; e < p.E; e += 32) {
+        const unsigned long long addr = p.wtab[e];
+        int blk = -1;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          if (addr >= p.base[i] && addr < p.base[i] + p.bytes * unsigned(p.count[i]))
+            blk = int((addr - p.base[i]) / p.bytes) + i * kStaging;
+        ctl->block[e] = blk;
+      }
+    }
     __syncwarp();
     int cnt[3], sum = 0, wide = 0;
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       const int pos = lane * 3 + j, s = nseg - 1 - pos;
-      const int rows = pos < nseg ? ctl->off[s + 1] - ctl->off[s] : 0;
-      bad |= rows > 0 && !in_mask(p.wmask, s);  // a selected expert without weights
+      int rows = pos < nseg ? ctl->off[s + 1] - ctl->off[s] : 0;
+      bool weights = rows > 0 && in_mask(p.wmask, s);
+      if constexpr (CACHED) {
+        if (rows > 0 && !rows_in_phase(p, s)) rows = 0;
+        if (rows > 0 && s < p.E) weights = ctl->block[s] >= 0;
+      }
+      bad |= rows > 0 && !weights;  // a selected expert without weights
       cnt[j] = token_tiles(rows) * p.mtiles;
       sum += cnt[j];
       wide = max(wide, tile_tokens(rows));
@@ -285,15 +345,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const CUtensorMap* mw = &p.w[t.seg];
         const CUtensorMap* mx = (sx ? p.sx : p.x) + (half / 16 - 1);
         const int nkb = p.kblocks;
+        int block = -1;  // of the maps over all of the cache's blocks
+        if constexpr (CACHED) {
+          if (t.seg < p.E) {
+            block = ctl->block[t.seg];
+            mw = &p.blocks[block >= kStaging ? 1 : 0];
+            block -= block >= kStaging ? kStaging : 0;
+          }
+        }
         int kb = 0;
         for (; kb < nkb; ++kb) {
           if (!mbar_wait_cl(&ctl->empty[s], ph ^ 1u, abort, p.err)) break;
           const uint32_t sa = base + uint32_t(s * stage_bytes), fb = fb0 + uint32_t(s) * 8u;
           if (leader) mbar_expect_tx(&ctl->full[s], bytes);
-          if constexpr (EPI == EPI_SWIGLU)
+          if (CACHED && block >= 0) {
+            if constexpr (EPI == EPI_SWIGLU)
+              tma_load_5d_pair(sa, mw, kb * BK, 0, 0, mrow * 4, block, fb);
+            else
+              tma_load_3d_pair(sa, mw, kb * BK, mrow * 128, block, fb);
+          } else if constexpr (EPI == EPI_SWIGLU) {
             tma_load_4d_pair(sa, mw, kb * BK, 0, 0, mrow * 4, fb);
-          else
+          } else {
             tma_load_2d_pair(sa, mw, kb * BK, mrow * 128, fb);
+          }
           tma_load_2d_pair(sa + kABytes, mx, kb * BK, xrow, fb);
           if (issued < stages) ++issued;
           if (++s == stages) {
@@ -457,7 +531,7 @@ bool encode(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims,
             const cuuint64_t* strides, const cuuint32_t* box) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  const cuuint32_t es[4] = {1, 1, 1, 1};
+  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, cuuint32_t(rank), const_cast<void*>(base), dims,
             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -560,14 +634,45 @@ bool fill_lora(RowsLoraParams& p, const FfnArgs& a, int mcap, int stage, int spl
   return true;
 }
 
+// The cache's blocks: encode_gate_up's and encode_rows' maps with the block as one dimension more.
+bool fill_cache(RowsCacheParams& p, const FfnArgs& a, const CacheBlocks& c, int stage) {
+  const uint64_t d = uint64_t(a.d), w = uint64_t(a.w);
+  for (int i = 0; i < 2; ++i) {
+    p.base[i] = reinterpret_cast<unsigned long long>(c.base[i]);
+    p.count[i] = c.count[i];
+    if (c.count[i] >= kStaging) return false;
+    if (c.count[i] == 0) continue;
+    const cuuint64_t n = cuuint64_t(c.count[i]), bytes = c.bytes;
+    const char* base = static_cast<const char*>(c.base[i]);
+    if (stage == 1) {
+      const cuuint64_t dims[5] = {d, 16, 2, w / 16, n}, strides[4] = {d * 2, w * d * 2, 16 * d * 2, bytes};
+      const cuuint32_t box[5] = {BK, 16, 2, 4, 1};
+      if (!encode(&p.blocks[i], base, 5, dims, strides, box)) return false;
+    } else {
+      const cuuint64_t dims[3] = {w, d, n}, strides[2] = {w * 2, bytes};
+      const cuuint32_t box[3] = {BK, 128, 1};
+      if (!encode(&p.blocks[i], base + 2 * w * d * 2, 3, dims, strides, box)) return false;
+    }
+  }
+  p.bytes = c.bytes;
+  p.wtab = a.wtab;
+  p.ready = a.ready;
+  p.phase = a.phase;
+  return true;
+}
+
 template <int EPI, typename P>
-cudaError_t run(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s, int split) {
+cudaError_t run(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s, int split,
+                const CacheBlocks* cache = nullptr) {
   P p;
   memset(&p, 0, sizeof(p));
   const int stage = EPI == EPI_SWIGLU ? 1 : 2;
   if (!fill(p, a, xp, mcap, stage)) return cudaErrorInvalidValue;
-  if constexpr (sizeof(P) == sizeof(RowsLoraParams)) {
+  if constexpr (std::is_same_v<P, RowsLoraParams>) {
     if (!fill_lora(p, a, mcap, stage, split)) return cudaErrorInvalidValue;
+  }
+  if constexpr (std::is_same_v<P, RowsCacheParams>) {
+    if (!fill_cache(p, a, *cache, stage)) return cudaErrorInvalidValue;
   }
   return launch_rows<EPI, P>(p, num_sms, s);
 }
@@ -583,6 +688,12 @@ cudaError_t launch_ffn_rows(const FfnArgs& a, const void* xp, int mcap, int num_
   if (e != cudaSuccess || !(stages & 2)) return e;
   return a.lrank > 0 ? run<EPI_F32, RowsLoraParams>(a, xp, mcap, num_sms, s, split)
                      : run<EPI_F32, RowsParams>(a, xp, mcap, num_sms, s, split);
+}
+
+cudaError_t launch_ffn_rows_cached(const FfnArgs& a, const CacheBlocks& cache, const void* xp, int mcap,
+                                   int num_sms, cudaStream_t s) {
+  const cudaError_t e = run<EPI_SWIGLU, RowsCacheParams>(a, xp, mcap, num_sms, s, 1, &cache);
+  return e != cudaSuccess ? e : run<EPI_F32, RowsCacheParams>(a, xp, mcap, num_sms, s, 1, &cache);
 }
 
 }  // namespace mcft

@@ -284,6 +284,14 @@ bool tc_pair_tiles(int T, int K, int E, int lrank);
 // split: bf16 halves of the LoRA middle vectors (u13 / u2 as launch_lora_down_tiles wrote them).
 cudaError_t launch_ffn_rows(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s,
                             int stages, int split);
+// The same for a cached forward: routed weights from the cache's blocks by a.wtab, the segments of a.phase.
+struct CacheBlocks {
+  const void* base[2];  // the layer's slots, the staging buffers
+  int count[2];
+  size_t bytes;         // of a block
+};
+cudaError_t launch_ffn_rows_cached(const FfnArgs& a, const CacheBlocks& cache, const void* xp, int mcap,
+                                   int num_sms, cudaStream_t s);
 struct CombineArgs {
   const float* o;
   const float* gate;
