@@ -140,8 +140,7 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   // The weight rows on M (gemm_rows.cu) unless the 256-row token tiles were asked for (gemm_tc.cu).
   // Whole passes, 128-row token tiles (removed) against gemm_rows: Mixtral shape at T = 2000 953 / 952
   // us, 4096 1940 / 1875, 8192 3753 / 3675, all 8 experts kept at 4096 2080 / 1947; DeepSeek-V2-Lite
-  // shape at 4096 641 / 478. The choice must not depend on adapters: mcft_gate_grad reads the
-  // workspace of a forward without knowing whether it had any.
+  // shape at 4096 641 / 478.
   L.rows = L.tc && !pair;
   L.split = aligned ? 1 : 2;
   L.pad = pair ? 256 : 1;
@@ -152,12 +151,14 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   L.cnt = o;  o = align256(o + sizeof(int) * nseg);
   L.off = o;  o = align256(o + sizeof(int) * (nseg + 1));
   L.pos = o;  o = align256(o + sizeof(int) * size_t(T) * K);
-  L.perm = o; o = align256(o + sizeof(int) * size_t(L.mcap));
   L.done = o; o = align256(o + sizeof(int) * (nseg + kClaimSlots));
-  L.xp = o;   o = align256(o + (L.tc && !compact ? size_t(L.mcap) * d * 2 : 0));
-  L.h = o;    o = align256(o + size_t(L.mcap) * w * (dtype == MCFT_BF16 ? 2 : 4));
-  if (compact) L.xp = o;
+  // Up to o, places depend on the layer and the batch alone and not on the rows' padding, which adapters and
+  // the tile shape decide: mcft_gate_grad finds the outputs without knowing what the forward had.
   L.o = o;    o = align256(o + size_t(L.ks) * L.mcap * d * 4);
+  L.xp = compact ? L.o : o;
+  if (!compact) o = align256(o + (L.tc ? size_t(L.mcap) * d * 2 : 0));
+  L.perm = o; o = align256(o + sizeof(int) * size_t(L.mcap));
+  L.h = o;    o = align256(o + size_t(L.mcap) * w * (dtype == MCFT_BF16 ? 2 : 4));
   L.u13 = o;  o = align256(o + size_t(L.mcap) * 2 * lrank * 4);
   L.u2 = o;   o = align256(o + size_t(L.mcap) * lrank * 4);
   L.total = o;
@@ -887,13 +888,15 @@ mcft_status mcft_gate_grad(const mcft_layer_desc* desc, const void* dy, int T, c
   if (reinterpret_cast<uintptr_t>(dy) & 15u) return fail(MCFT_ERR_INVALID, "dy must be 16-byte aligned");
   const WsLayout L =
       ws_layout(desc->d, desc->E, desc->K, desc->w, desc->n_shared, desc->dtype, T);
-  if (ws_bytes < L.o + size_t(L.ks) * L.mcap * desc->d * 4)
+  // at least the rows without padding; the kernel compares the rows that the forward laid out
+  const size_t row = size_t(L.ks) * desc->d * 4;
+  if (ws_bytes < L.o + size_t(T) * (desc->K + desc->n_shared) * row)
     return fail(MCFT_ERR_INVALID, "workspace of %zu bytes is not a forward workspace for T = %d",
                 ws_bytes, T);
   const char* ws = static_cast<const char*>(workspace);
   GateGradArgs a{dy, reinterpret_cast<const float*>(ws + L.o), reinterpret_cast<const int*>(ws + L.pos),
-                 reinterpret_cast<const WsHeader*>(ws + L.hdr), size_t(L.mcap) * desc->d, T, desc->K,
-                 desc->d, L.ks, dgate};
+                 reinterpret_cast<const WsHeader*>(ws + L.hdr), size_t(L.mcap) * desc->d,
+                 (ws_bytes - L.o) / row, device_error_word(), T, desc->K, desc->d, L.ks, dgate};
   cudaError_t e = launch_gate_grad(a, desc->dtype, stream);
   if (e != cudaSuccess) return cuda_fail(e, "gate gradient kernel launch");
   return MCFT_OK;

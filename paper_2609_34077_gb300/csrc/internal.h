@@ -85,7 +85,7 @@ struct WsLayout {
                   // for CTA-pair tiles)
   int mcap;       // capacity in permuted rows
   int ks;         // partial planes of o (contraction split of the decode GEMM2)
-  size_t hdr, cnt, off, pos, perm, done, xp, h, o, u13, u2, total;
+  size_t hdr, cnt, off, pos, done, o, xp, perm, h, u13, u2, total;
 };
 // compact: xp takes o's memory (GEMM13 has read the permuted activations when GEMM2, which writes o, starts).
 WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0,
@@ -424,6 +424,8 @@ struct GateGradArgs {
   const int* pos;      // forward workspace: permuted row of each assignment
   const WsHeader* hdr;
   size_t o_plane;
+  size_t rows;         // most rows of o that the workspace can hold
+  unsigned* err;
   int T, K, d, ks;
   float* dgate;        // [T, K] out
 };

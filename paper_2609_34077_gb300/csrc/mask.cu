@@ -110,6 +110,10 @@ template <typename TY>
 __global__ void __launch_bounds__(256) gate_grad_kernel(const __grid_constant__ GateGradArgs a) {
   pdl_wait();
   if (a.hdr->abort) return;
+  if (size_t(a.hdr->mrows) > a.rows) {  // not the whole workspace of that forward
+    if (threadIdx.x == 0) set_error(a.err, kErrInvalid);
+    return;
+  }
   const int lane = threadIdx.x & 31;
   const int n = a.T * a.K;
   for (int i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {

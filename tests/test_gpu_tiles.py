@@ -100,3 +100,36 @@ def test_workspace_sized_for_one_cta_tiles_is_rejected_under_pairs():
     finally:
         M.mcft_set_tc_tiles(M.MCFT_TC_TILES_ONE_CTA)
     M.mcft_device_error()
+
+
+@pytest.mark.parametrize("rank", [0, 8, 16])
+def test_gate_gradient_under_pairs(rank):
+    """The gate gradient of a forward with and without adapters, whose segments are laid out with other
+    padding under the pair mode: the default mode's bits. A workspace cut off before the padded rows is
+    reported."""
+    shape = I.LayerShape("pair-grad", d=256, E=4, K=2, w=128, n_shared=1, gate=I.GATE_RENORM, dtype=I.BF16,
+                         cache_slots=2, keep=4)
+    T = 1024
+    desc, x, idx, gate, experts, shared = _case(shape, T, 140, hot=[1], p_hot=0.5)
+    dy = I.hidden_iid(141, shape, T, tag="dy").to(DEV)
+    ad = [I.lora_block(142, shape, e, rank).to(DEV) for e in range(4)] if rank else None
+    sad = [I.lora_block(142, shape, ("shared", 0), rank).to(DEV)] if rank else None
+    out = []
+    try:
+        for mode in (M.MCFT_TC_TILES_ONE_CTA, M.MCFT_TC_TILES_CTA_PAIR):
+            M.mcft_set_tc_tiles(mode)
+            n = M.mcft_moe_workspace_size_lora(desc, rank, T) if rank else M.mcft_moe_workspace_size(desc, T)
+            ws = torch.empty(n, dtype=torch.uint8, device=DEV)
+            if rank:
+                M.mcft_moe_forward_lora(desc, x, idx, gate, experts, shared, ad, sad, rank, 2.0, workspace=ws)
+            else:
+                M.mcft_moe_forward(desc, x, idx, gate, experts, shared, workspace=ws)
+            out.append(M.mcft_gate_grad(desc, dy, ws))
+            M.mcft_device_error()
+        if not rank:  # room for the 3 T rows, but not for their padding
+            with pytest.raises(M.MCFTError):
+                M.mcft_gate_grad(desc, dy, ws[:3 * T * shape.d * 4 + (16 << 10)])
+                M.mcft_device_error()
+    finally:
+        M.mcft_set_tc_tiles(M.MCFT_TC_TILES_ONE_CTA)
+    assert out[0].abs().max() > 0 and torch.equal(out[0], out[1])
