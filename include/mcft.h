@@ -150,7 +150,8 @@ mcft_status mcft_moe_forward(const mcft_layer_desc* desc, const void* x, int T, 
  *   lora_rank    8 or 16 (MCFT_ERR_UNSUPPORTED otherwise); lora_scale finite
  * The workspace needs mcft_moe_workspace_size_lora(desc, lora_rank, T) bytes. On the tensor-core
  * path (bf16, T > 64) the down projections are skinny GEMMs on the tensor cores and the up
- * projections one extra k-block of each adapted tile of the expert GEMMs; on the decode and fp32
+ * projections extra k-blocks of each adapted tile of the expert GEMMs, with s (A v) rounded to bf16
+ * where d % 256 == 0 and w % 128 == 0 and to fp32 at other sizes; on the decode and fp32
  * paths a small kernel computes A v and the up projections are added as the expert GEMV finishes
  * each output. Adapters that add nothing (B = 0, or none) give mcft_moe_forward's result bit for
  * bit. No dropout (a forward whose output is compared). */

@@ -142,7 +142,9 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   // us, 4096 1940 / 1875, 8192 3753 / 3675, all 8 experts kept at 4096 2080 / 1947; DeepSeek-V2-Lite
   // shape at 4096 641 / 478.
   L.rows = L.tc && !pair;
-  L.split = aligned ? 1 : 2;
+  // The middle vectors of adapters: bf16 where the tensor cores have always taken them (d % 256 == 0 and w %
+  // 128 == 0), and all of fp32 where they were fp32 before these kernels took the other sizes.
+  L.split = aligned ? 1 : 3;
   L.pad = pair ? 256 : 1;
   const int nseg = E + S;
   L.mcap = T * K + S * T + nseg * (L.pad - 1);
@@ -161,6 +163,7 @@ WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lran
   L.h = o;    o = align256(o + size_t(L.mcap) * w * (dtype == MCFT_BF16 ? 2 : 4));
   L.u13 = o;  o = align256(o + size_t(L.mcap) * 2 * lrank * 4);
   L.u2 = o;   o = align256(o + size_t(L.mcap) * lrank * 4);
+  if (L.tc) L.u2 = L.u13;  // (three bf16 parts fill both; u13 has been read when u2 is written)
   L.total = o;
   return L;
 }

@@ -53,7 +53,7 @@
 //
 // With LoRA adapters (Section 3.2, Stage 2) an adapted tile appends p.nx k-blocks of one MMA each,
 // D += B' U^T: for GEMM13 B' is B1 on the gate rows (zeros on the up rows) with U = s A1 x, then B3 on
-// the up rows with U = s A3 x (and, if kept, the low halves of U against the same B'); for GEMM2
+// the up rows with U = s A3 x (and, if kept, the other bf16 parts of U against the same B'); for GEMM2
 // B' = B2, U = s A2 h. The zeros are TMA out-of-bounds fill: the adapter matrices are r columns wide
 // under boxes of 64, and the W1 / W3 dimension of the box is one plane long, entered at 0 or at -1.
 //
@@ -81,7 +81,6 @@ constexpr int kMaxStages = 10;
 constexpr int kABytes = 128 * BK * 2;         // a CTA's weight rows of a stage
 constexpr int kRingBytes = 7 * (kABytes + (kTileTok / 2) * BK * 2);
 constexpr int kTmemCols = 2 * kTileTok;
-constexpr int kMaxExtra = 4;
 // instruction descriptor without N: D fp32, A and B bf16, both K-major, M = 256
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(256 >> 4) << 24);
 
@@ -99,7 +98,7 @@ struct RowsParams {
   int nseg, E, kblocks, mtiles, ldo, group_x, use_sx;
 };
 struct RowsLoraParams : RowsParams {
-  CUtensorMap u[kMaxExtra][kUBoxes];  // U of each extra k-block
+  CUtensorMap u[kUBoxes];            // U [rows, extra k-blocks, r]
   CUtensorMap lb[2][kMaxSeg];        // GEMM13: B1, B3; GEMM2: B2
   uint32_t lmask[3];                 // segments with an adapter
   int nx;
@@ -391,7 +390,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int b = kUBoxes - 1; b >= 0; --b)
               if (half & (16 << b)) {
-                tma_load_2d_pair(sa + kABytes + uint32_t(r) * (BK * 2), &p.u[e][b], 0,
+                tma_load_3d_pair(sa + kABytes + uint32_t(r) * (BK * 2), &p.u[b], 0, e,
                                  t.row0 + int(rank) * half + r, fb);
                 r += 16 << b;
               }
@@ -610,17 +609,17 @@ bool fill(RowsParams& p, const FfnArgs& a, const void* xp, int mcap, int stage) 
   return true;
 }
 
-// The adapters of one GEMM. U planes of r columns side by side: GEMM13 [s A1 x | s A3 x] (then their
-// low halves), GEMM2 s A2 h (then its low half); 16-byte rows and offsets for r = 8 and 16.
+// The adapters of one GEMM. U planes of r columns side by side: GEMM13 [s A1 x | s A3 x], GEMM2 s A2 h, then
+// the same of each further bf16 part; 16-byte rows and offsets for r = 8 and 16.
 bool fill_lora(RowsLoraParams& p, const FfnArgs& a, int mcap, int stage, int split) {
   const LoraOffsets lo = lora_offsets(a.d, a.w, a.lrank);
   const uint64_t r = uint64_t(a.lrank);
   p.nx = (stage == 1 ? 2 : 1) * split;
-  const char* u = reinterpret_cast<const char*>(stage == 1 ? a.u13 : a.u2);
-  for (int e = 0; e < p.nx; ++e)
-    for (int b = 0; b < kUBoxes; ++b)
-      if (!encode_rows(&p.u[e][b], u + size_t(e) * r * 2, r, uint64_t(mcap), p.nx * r, 16u << b))
-        return false;
+  const cuuint64_t nx = cuuint64_t(p.nx), dims[3] = {r, nx, uint64_t(mcap)}, strides[2] = {r * 2, nx * r * 2};
+  for (int b = 0; b < kUBoxes; ++b) {
+    const cuuint32_t box[3] = {BK, 1, 16u << b};
+    if (!encode(&p.u[b], stage == 1 ? a.u13 : a.u2, 3, dims, strides, box)) return false;
+  }
   for (int s = 0; s < a.nseg; ++s) {
     const char* blk = reinterpret_cast<const char*>(a.lblk[s]);
     if (!blk || !a.wblk[s]) continue;

@@ -80,7 +80,7 @@ struct WsLayout {
   bool tc;        // tensor-core path (bf16, large T)
   bool decode;    // bf16 decode path (T <= 64)
   bool rows;      // tensor-core path with the weight rows on M (gemm_rows.cu): segments unpadded
-  int split;      // bf16 halves that keep a LoRA middle vector on that path
+  int split;      // bf16 parts that keep a LoRA middle vector on that path
   int pad;        // rows per segment are padded to a multiple of this (TC path: 1, 128, or 256
                   // for CTA-pair tiles)
   int mcap;       // capacity in permuted rows
@@ -125,7 +125,7 @@ struct LoraDownArgs {
   float* u;              // output [mcap, ustride]
   int ustride;
   float scale;           // tiles: U is scaled by it (lora_down leaves the scale to the epilogues)
-  int split;             // tiles: 1 = bf16 U, 2 = bf16 high and low halves
+  int split;             // tiles: 1 = bf16 U, 3 = all of the fp32 value as three bf16 parts
 };
 // The same on the tensor cores for large bf16 batches (U in bf16, see lora.cu), 16 rows per CTA.
 cudaError_t launch_lora_down_tiles(const LoraDownArgs& a, int outs, int mcap, int num_sms, cudaStream_t s);
@@ -281,7 +281,7 @@ cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, i
                           cudaStream_t s, int stages = 3);
 bool tc_pair_tiles(int T, int K, int E, int lrank);
 // The expert GEMMs with the weight rows on M (gemm_rows.cu): any d and w, unpadded segments.
-// split: bf16 halves of the LoRA middle vectors (u13 / u2 as launch_lora_down_tiles wrote them).
+// split: bf16 parts of the LoRA middle vectors (u13 / u2 as launch_lora_down_tiles wrote them).
 cudaError_t launch_ffn_rows(const FfnArgs& a, const void* xp, int mcap, int num_sms, cudaStream_t s,
                             int stages, int split);
 // The same for a cached forward: routed weights from the cache's blocks by a.wtab, the segments of a.phase.

@@ -3,9 +3,9 @@
 //
 // Each adapted projection is W v + s B (A v) with A [r, in], B [out, r], s = alpha / r. The large
 // term W v runs in the expert GEMM / GEMV kernels, which also add s B u in their epilogues (r
-// multiply-adds per output). On the decode and fp32 paths this kernel computes the small middle
-// vectors u = A v for every permuted row whose segment has an adapter (the tcgen05 path projects
-// its gathered rows on the tensor cores and takes A2 h from GEMM13's epilogue instead):
+// multiply-adds per output). On the decode and fp32 paths lora_down_kernel computes the small middle
+// vectors u = A v for every permuted row whose segment has an adapter (the tensor-core path has
+// lora_down_tile_kernel below, and adds B u as further k-blocks of its GEMMs):
 //   stage 13: u[q] = [A1 x ; A3 x]     (2r values; x = the row's token, or the gathered row)
 //   stage 2:  u[q] = A2 h_q            (r values; h = the SwiGLU activation of the row)
 // One warp per row: lanes walk the input in 16-byte chunks, each chunk is dotted with the R rows
@@ -88,8 +88,9 @@ __global__ void __launch_bounds__(kWarps * 32) lora_down_kernel(const __grid_con
 }
 
 // The down projections of the tensor-core path: U = s (A v) in bf16 for the rows of every segment
-// with an adapter, [rows, NT * 8] ([s A1 x | s A3 x] or s A2 h), or with `split` [rows, 2 * NT * 8]: the
-// bf16 high halves, then what they leave of the fp32 value, again in bf16. A skinny GEMM bound by
+// with an adapter, [rows, NT * 8] ([s A1 x | s A3 x] or s A2 h), or with split = 3 [rows, 3 * NT * 8]: bf16
+// of the fp32 values, of what that leaves of them, and of what is left then, which together hold all 24 bits.
+// A skinny GEMM bound by
 // reading v once: as in the router's tiles, a CTA takes 16 rows of one segment and its 8 warps one
 // contraction slice each (mma.sync m16n8k16, U 32-element chunks of every operand in flight per
 // lane), so 2000 rows are 125 CTAs; partial sums are added in shared memory in slice order.
@@ -130,7 +131,6 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
   __syncthreads();
   const int nch = a.K / 32;
   const int c0 = warp * nch / kWarps, c1 = (warp + 1) * nch / kWarps;
-  const size_t krow = size_t(a.K) * 2;
   for (int tile = blockIdx.x; tile < s_first[nseg]; tile += gridDim.x) {
     int lo = 0, hi = nseg - 1;  // the last segment whose first tile is <= tile: it is not empty
     while (lo < hi) {
@@ -194,10 +194,14 @@ __global__ void __launch_bounds__(kWarps * 32, 2)
 #pragma unroll
       for (int k = 1; k < kWarps; ++k) v += part[k][r][o];
       v *= a.scale;
-      uint16_t* u = reinterpret_cast<uint16_t*>(a.u) + size_t(q0 + r) * (a.split * NT * 8);
-      const uint16_t h = f2bf(v);
-      u[o] = h;
-      if (a.split > 1) u[NT * 8 + o] = f2bf(v - bf16lo(h));
+      uint16_t* u = reinterpret_cast<uint16_t*>(a.u) + size_t(q0 + r) * (a.split * NT * 8) + o;
+      const bool finite = fabsf(v) < INFINITY;
+      for (int i = 0; i < a.split; ++i) {
+        uint16_t h = f2bf(v);
+        if (finite && a.split > 1 && (h & 0x7fff) == 0x7f80) h -= 1;  // rounded past the largest number
+        u[i * NT * 8] = h;
+        v = finite ? v - bf16lo(h) : 0.f;
+      }
     }
   }
 }
