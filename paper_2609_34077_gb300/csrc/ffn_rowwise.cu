@@ -413,16 +413,26 @@ cudaError_t launch_combine_typed(const CombineArgs& a, cudaStream_t s) {
   }
 }
 
+// Rows an expert averages from which the 64-token tiles (ffn_tile.cu) win. They take whole tiles' time however
+// few their rows, and with few experts there are fewer tiles than SMs, so the line lies higher there, and
+// higher yet where a tile's contraction is long. Graph-replayed forwards, row-wise / tiles, at 12, 16 and 20 rows:
+// d 256, w 512: 4 experts 0.89, 1.05, 1.27, 8 experts 1.09, 1.29, 1.46, 32 experts 1.32, 1.71, 2.00; d 512, w 1024:
+// 4 experts 0.62-0.80, 0.88-1.00, 1.11-1.22, 16 experts 1.02, 1.15, 1.50, 32 experts 1.00, 1.30, 1.58; d 512, w 512, 8
+// and 16 experts: 0.78, 0.79, 1.22 and 0.91, 1.11, 1.35; d 384, w 768, 16 experts 0.88, 1.01, 1.27; d 128, w 128, 4
+// experts 1.17, 1.26, 1.50; d 64, w 1024, 4 experts 0.90-1.05, 1.09, 1.33.
+// A function of the layer only, so every phase and path of a call takes the same kernel.
+int tile_min_rows(int d, int w, int E) {
+  if (E >= 32 || (d <= 128 && w <= 256)) return 12;
+  if (d < 384) return E >= 16 || (E >= 8 && w < 1024) ? 12 : 16;
+  return E >= 16 ? 16 : 20;
+}
+
 }  // namespace
 
 cudaError_t launch_ffn_rowwise(const FfnArgs& a, int dtype, int num_sms, cudaStream_t s, int stages) {
   if (dtype != MCFT_F32) return cudaErrorInvalidValue;  // bf16 layers use the decode or TC path
-  // Rows an expert averages from which the 64-token tiles (ffn_tile.cu) win. Whole passes, row-wise
-  // against tiles: d 512, w 1024, 32 experts: 100 / 171 us at 4 rows, 142 / 177 at 8, 427 / 211 at 32;
-  // d 256, w 512: 64 experts 83 / 96 at 4, 117 / 100 at 8, 8 experts 348 / 60 at 128 (512 tokens).
-  // A function of the layer and the batch only, so every phase and path of a call takes the same.
-  constexpr int kTileMinRows = 12;
-  if (size_t(a.T) * a.K >= size_t(kTileMinRows) * a.E) return launch_ffn_tile(a, num_sms, s, stages);
+  if (size_t(a.T) * a.K >= size_t(tile_min_rows(a.d, a.w, a.E)) * a.E)
+    return launch_ffn_tile(a, num_sms, s, stages);
   return launch_rowwise_typed<float>(a, num_sms, s, stages);
 }
 
