@@ -141,9 +141,9 @@ struct PermuteArgs {
   int* perm;   // [mcap] token of each permuted row, -1 for padding
   unsigned* err;
   int* done;   // [E+S + kClaimSlots] progress and claim counters of the fused decode FFN, zeroed here
-  int spread;  // T > kPermDecodeT: launch_spread follows and writes the routed rows of perm
+  int spread;  // launch_spread follows and writes the routed rows of perm
 };
-constexpr int kPermDecodeT = 64;  // up to this many tokens one CTA permutes
+constexpr int kPermDecodeT = 64;  // up to this many tokens (or 1024 assignments) one CTA permutes
 cudaError_t launch_permute(const PermuteArgs& a, cudaStream_t s);
 
 struct SpreadArgs {

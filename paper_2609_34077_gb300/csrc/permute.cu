@@ -158,7 +158,9 @@ __global__ void __launch_bounds__(kThreads) permute_kernel(const __grid_constant
 // and places it. A chain of dependent steps bounds it, not the 100 KB of ids. ncu, GB300: T = 4096 with
 // K = 6 8.1 us against 15.4 for a count, a scan and a scatter launch (K = 2: 5.5 / 12), T = 16384 with K = 6
 // 16.7 / 17.2, and 1200 assignments (T = 200) 6.2 us against 8.6 for the one-CTA kernel above, which walks
-// 1024 assignments at a time; at decode sizes that kernel stays: it lets the FFN start beside it.
+// 1024 assignments at a time. Up to one such walk that kernel is the faster one: whole forwards of small layers,
+// cluster / one CTA: 65 assignments 16.9 / 16.0 us, 512 17.8 / 17.0, 1024 18.7 / 18.3, 1500 18.9 / 20.1 (64 experts).
+// At decode sizes it stays too: it lets the FFN start beside it.
 constexpr int kPermCtas = 8;
 constexpr int kPermWarps = kThreads / 32;
 constexpr int kPermAhead = 4;  // rounds of ids loaded together
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(kSpreadWarps * 32) spread_kernel(const __grid_
 cudaError_t launch_permute(const PermuteArgs& a, cudaStream_t s) {
   prof_begin(kProfPermute, s);
   cudaError_t e;
-  if (a.T <= kPermDecodeT) {
+  if (a.T <= kPermDecodeT || a.T * a.K <= kThreads) {
     e = launch_pdl(permute_kernel, dim3(1), dim3(kThreads), 0, s, a);
   } else {
     e = launch_pdl(permute_cluster_kernel, dim3(kPermCtas), dim3(kThreads), 0, s, a);
