@@ -313,7 +313,7 @@ mcft_status mcft_test_inject(int fail_pinned_allocs, int fail_expert_copies,
 
 mcft_status mcft_set_tc_tiles(int mode) {
   if (mode != MCFT_TC_TILES_ONE_CTA && mode != MCFT_TC_TILES_CTA_PAIR)
-    return fail(MCFT_ERR_INVALID, "tile mode %d is neither one-CTA (0) nor CTA-pair (1)", mode);
+    return fail(MCFT_ERR_INVALID, "tile mode %d is neither the default (0) nor CTA-pair token tiles (1)", mode);
   g_tc_tiles.store(mode);
   return MCFT_OK;
 }

@@ -547,7 +547,8 @@ __device__ bool wait_landed(const FfnArgs& a, unsigned epoch, int e, size_t off,
 // kernel. Two CTAs of 256 threads at up to 128 registers fill an SM, so a fetch kernel needs slots kept
 // free for it; up to 8 tokens also fit 96 registers without spills, which leaves room for one of its
 // 40-register CTAs beside two of these, so that build takes every slot. Three-layer DeepSeek-V2-Lite
-// chain with prefetch 2: T = 1 206 -> 198 us, T = 2 297 -> 290, but T = 4, which the link bounds, 857 / 864.
+// chain with prefetch 2, medians of four alternating runs that differ by under 1 us: T = 1 206.0 -> 195.6 us, T = 2
+// 297.6 -> 289.0; T = 4, which the link bounds, 857 / 864.
 // Alone 96 registers are slower (T = 1 44.1 / 44.7 us, a chain without prefetch 157 / 162).
 enum { kPlain = 0, kFetch = 1 };
 constexpr int kBesideMaxT = 2;

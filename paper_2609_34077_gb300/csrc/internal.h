@@ -81,8 +81,7 @@ struct WsLayout {
   bool decode;    // bf16 decode path (T <= 64)
   bool rows;      // tensor-core path with the weight rows on M (gemm_rows.cu): segments unpadded
   int split;      // bf16 parts that keep a LoRA middle vector on that path
-  int pad;        // rows per segment are padded to a multiple of this (TC path: 1, 128, or 256
-                  // for CTA-pair tiles)
+  int pad;        // rows per segment are padded to a multiple of this (1, or 256 for CTA-pair token tiles)
   int mcap;       // capacity in permuted rows
   int ks;         // partial planes of o (contraction split of the decode GEMM2)
   size_t hdr, cnt, off, pos, done, o, xp, perm, h, u13, u2, total;
@@ -90,7 +89,8 @@ struct WsLayout {
 // compact: xp takes o's memory (GEMM13 has read the permuted activations when GEMM2, which writes o, starts).
 WsLayout ws_layout(int d, int E, int K, int w, int S, int dtype, int T, int lrank = 0,
                    bool compact = false);
-// Layer sizes that fill the 128 x 256 tiles of gemm_tc.cu.
+// Layer sizes that fill the CTA-pair token tiles (128 outputs of GEMM13, 256 of GEMM2). Above 64 tokens the
+// cached forward refuses them, and adapters' middle vectors are bf16 there.
 inline bool tc_aligned(int d, int w) { return d % 256 == 0 && w % 128 == 0; }
 
 // LoRA adapter block of one expert (layer dtype, row-major), element offsets for rank r:
@@ -275,8 +275,8 @@ cudaError_t launch_ffn_tile(const FfnArgs& a, int num_sms, cudaStream_t s, int s
 cudaError_t launch_ffn_decode(const FfnArgs& a, int num_sms, cudaStream_t s, int stages = 3,
                               int reserved = 0);  // bf16, T <= 64
 int decode_ksplit(int T);  // contraction split of the decode GEMM2 for T tokens
-// pad: rows per segment of the permutation, 256: the CTA-pair tiles, which
-// tc_pair_tiles chooses, when selected, for layers without adapters whose routed experts average >= 512 rows).
+// pad: rows per segment of the permutation, 256 (tc_pair_tiles says which layers take these tiles when they are
+// selected: without adapters, and routed experts that average at least 512 rows).
 cudaError_t launch_ffn_tc(const FfnArgs& a, const void* xp, int mcap, int pad, int num_sms,
                           cudaStream_t s, int stages = 3);
 bool tc_pair_tiles(int T, int K, int E, int lrank);

@@ -1,8 +1,8 @@
 // Token permutation by expert: histogram, exclusive scan of padded segment sizes, and a stable
-// scatter (assignments keep their (t, k) order inside each expert), plus the row gather that builds
-// the permuted activation matrix for the tensor-core path. Segments E..E+S-1 hold the shared
+// scatter (assignments keep their (t, k) order inside each expert), plus the spread of the activations
+// into the permuted matrix for the tensor-core path. Segments E..E+S-1 hold the shared
 // experts, which process every token (Section 3.1). The stable order defines the result uniquely,
-// so the one-CTA kernel (decode batches) and the cluster (large batches) write the same rows.
+// so the one-CTA kernel (decode and other small batches) and the cluster write the same rows.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -112,7 +112,7 @@ __device__ void fill_rows(const PermuteArgs& a, const int* offs, const int* len_
   }
 }
 
-// One CTA for the whole call (decode batches: a few microseconds).
+// One CTA for the whole call (decode batches, and up to 1024 assignments: a few microseconds).
 __global__ void __launch_bounds__(kThreads) permute_kernel(const __grid_constant__ PermuteArgs a) {
   pdl_wait();
   // the next launch (the decode FFN) may start now: before its own wait it reads only what was
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kThreads) permute_kernel(const __grid_constant
   fill_rows(a, offs, hist, tid, kThreads);
 }
 
-// Prefill-sized calls: the same permutation by one cluster of 8 CTAs. Each of its 256 warps takes a
+// Larger calls: the same permutation by one cluster of 8 CTAs. Each of its 256 warps takes a
 // contiguous stretch of the assignments and counts them per expert (its own row of counters, so no
 // atomics); the counters of a CTA's warps and then, over distributed shared memory, of the CTAs are
 // scanned per expert; every CTA scans the segment sizes for itself; and each warp walks its stretch again

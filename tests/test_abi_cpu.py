@@ -97,7 +97,7 @@ def test_test_inject_validation_without_gpu(libpath):
 def test_tc_tile_mode_without_gpu(libpath):
     """mcft_set_tc_tiles: only the two modes; under CTA-pair tiles a layer whose routed experts
     average >= 512 rows pads its segments to 256 rows (a larger workspace), a smaller one keeps
-    the one-CTA layout, and a layer with adapters always does."""
+    the default layout, and a layer with adapters always does."""
     import ctypes as C
     from paper_2609_34077_gb300 import inputs as I
     from paper_2609_34077_gb300 import mcft

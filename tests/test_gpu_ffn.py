@@ -139,7 +139,7 @@ def test_ffn_empty_and_bad_ids():
     M.mcft_device_error()
     # an id out of range: the device error word is set and y is left untouched (every decode
     # kernel variant: 1, 16 and 64 tokens; the tensor-core path; and 6000 assignments, which the
-    # chunked permutation handles)
+    # cluster permutation handles)
     for T in (1, 16, 64, 100, 3000):
         idx = torch.zeros((T, 2), dtype=torch.int32, device=DEV)
         idx[:, 1] = 1
@@ -167,9 +167,8 @@ def test_ffn_empty_and_bad_ids():
 @pytest.mark.parametrize("shape,T", [(SMALL_BF16, 2049), (SMALL_BF16, 2500), (SMALL_DS, 700)],
                          ids=["mix-4098", "mix-5000", "ds-4200"])
 def test_ffn_chunked_permutation(shape, T):
-    """Just above 4096 assignments the permutation runs in chunks (ragged: 820 to 1000
-    assignments each, shared-expert rows filled by every chunk's CTA); every output row matches
-    the oracle."""
+    """Some 4100 to 5000 assignments, shared out over the cluster permutation's warps in ragged
+    stretches (shared-expert rows filled by every CTA); every output row matches the oracle."""
     lw = weights(shape)
     x = I.hidden_iid(13, shape, T)
     idx, gate = _routing(shape, T, 13, hot=range(shape.keep))

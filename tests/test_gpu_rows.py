@@ -98,9 +98,10 @@ def test_adapters(d, w, rank):
 
 
 def test_large_batches_of_unaligned_sizes_elsewhere():
-    """d and w off the 128 x 256 tiles: the cached forward takes more than 64 tokens of them and its
-    workspace serves mcft_gate_grad, and the no-allocation entry point falls back to the smaller
-    decode layout when the batch needs more than its static array."""
+    """d and w off the 256 / 128 multiples: the cached forward takes more than 64 tokens of them and its
+    workspace serves mcft_gate_grad, and the no-allocation entry point serves batches whose workspace
+    is larger than its static array, with the permuted activations in the outputs' memory (their bits
+    against the plain forward's: test_gpu_same_bits.py)."""
     shape = _shape(320, 192, E=8, S=1)
     T, seed = 130, 220
     ids = _sized_ids(T, 2, 8, [40, 33])
@@ -119,7 +120,6 @@ def test_large_batches_of_unaligned_sizes_elsewhere():
     M.mcft_moe_forward(*args, workspace=ws2)
     dg2 = M.mcft_gate_grad(desc, dy, ws2)
     M.mcft_device_error()
-    # both compute <dy, F(x)> from bf16 h: the h of the two paths differ by its rounding at most
     assert ((dg - dg2).norm() / dg2.norm()).item() < 4 * 2.0 ** -8
     big = I.LayerShape("rows-noalloc", d=320, E=8, K=2, w=1728, n_shared=0, gate=I.GATE_RENORM,
                        dtype=I.BF16, cache_slots=4, keep=8)

@@ -1,7 +1,7 @@
 """The CTA-pair tile shape of the tensor-core expert GEMMs (mcft_set_tc_tiles): 256-row tiles whose
 MMAs run over the shared memory of a 2-CTA cluster, with segments padded to 256 rows. The same
-products are summed in the same order as on the one-CTA tiles, so the forward (Section 3.1, the
-gated sum of SwiGLU experts) must give the same bits; the one-CTA path is itself compared with the
+products are summed in the same order as on the default tiles, so the forward (Section 3.1, the
+gated sum of SwiGLU experts) must give the same bits; the default path is itself compared with the
 oracle on every row in test_gpu_layer.py, and one pair-tile forward is compared here too."""
 import numpy as np
 import pytest
@@ -82,7 +82,7 @@ def test_cta_pair_tiles_against_the_oracle_every_row():
 
 
 def test_small_layers_keep_one_cta_tiles():
-    """Routed experts averaging fewer than 512 rows keep the one-CTA tiles under the pair mode."""
+    """Routed experts averaging fewer than 512 rows keep the default tiles under the pair mode."""
     desc, x, idx, gate, experts, shared = _case(I.MIXTRAL, 1024, 131, keep=4)
     y1, _, ws1 = _forward(desc, x, idx, gate, experts, shared, M.MCFT_TC_TILES_ONE_CTA)
     y2, p2, ws2 = _forward(desc, x, idx, gate, experts, shared, M.MCFT_TC_TILES_CTA_PAIR)
