@@ -166,3 +166,63 @@ def test_stack_step_stays_in_bounds(T):
         M.mcft_stack_step(stack, x)
     M.mcft_device_error()
     gx.check("stack stream")
+
+
+# bf16 sizes off the 256 / 128 multiples, over 64 tokens: tensor cores with middle vectors in three parts, and
+# the cached forward on the same kernels
+ODD_BF16 = I.LayerShape("canary-odd", d=192, E=8, K=2, w=320, n_shared=1, gate=I.GATE_RENORM, dtype=I.BF16,
+                        cache_slots=3, keep=6)
+
+
+@pytest.mark.parametrize("rank", [8, 16])
+@pytest.mark.parametrize("T", [65, 300])
+def test_lora_forward_of_other_sizes_stays_in_bounds(rank, T):
+    shape = ODD_BF16
+    desc = M.desc_of(shape)
+    lw = I.layer_weights(75, shape)
+    x = I.hidden_iid(75, shape, T).to(DEV)
+    idx, gate = _ids(shape, T, 75)
+    lora = [I.lora_block(75, shape, e, rank).to(DEV) for e in range(shape.E)]
+    gws = Guarded(M.mcft_moe_workspace_size_lora(desc, rank, T))
+    gy = Guarded(T * shape.d * 2)
+    y = gy.view(torch.bfloat16, (T, shape.d))
+    M.mcft_moe_forward_lora(desc, x, idx, gate, [b.to(DEV) for b in lw.experts], [b.to(DEV) for b in lw.shared],
+                            lora, [I.lora_block(75, shape, ("shared", 0), rank).to(DEV)], rank=rank, scale=2.0,
+                            y=y, workspace=gws.view())
+    M.mcft_device_error()
+    gws.check("LoRA workspace")
+    gy.check("LoRA output")
+    assert bool(torch.isfinite(y.float()).all())
+
+
+@pytest.mark.parametrize("T", [65, 300])
+def test_cached_forward_of_other_sizes_stays_in_bounds(T):
+    """Also the plain forward's bits, with a prefetch before every other step."""
+    shape = ODD_BF16
+    desc = M.desc_of(shape)
+    lw = I.layer_weights(76, shape, pin=True)
+    cache = M.mcft_cache_create(1, shape.E, shape.cache_slots, shape.expert_bytes, lw.experts,
+                                max_assign=T * shape.K)
+    shared = [b.to(DEV) for b in lw.shared]
+    experts = [b.to(DEV) for b in lw.experts]
+    gws = Guarded(M.mcft_moe_workspace_size(desc, T))
+    gy = Guarded(T * shape.d * 2)
+    y = gy.view(torch.bfloat16, (T, shape.d))
+    compute, copy = torch.cuda.Stream(), torch.cuda.Stream()
+    for s in range(6):
+        x = I.hidden_iid(76 + s, shape, T).to(DEV)
+        idx, gate = _ids(shape, T, 76 + s)
+        nxt = _ids(shape, T, 77 + s)[0]
+        want = M.mcft_moe_forward(desc, x, idx, gate, experts, shared)
+        torch.cuda.synchronize()
+        M.mcft_cache_step(cache, 0, idx, stream=compute)
+        M.mcft_moe_forward_cached(desc, x, idx, gate, cache, 0, shared, y=y, workspace=gws.view(),
+                                  compute_stream=compute, copy_stream=copy)
+        if s % 2:  # for the next step, whose forward call fetches it
+            M.mcft_cache_prefetch(cache, 0, nxt, 2, stream=compute)
+        compute.synchronize()
+        copy.synchronize()
+        assert torch.equal(y, want), s
+    M.mcft_device_error()
+    gws.check("cached forward workspace")
+    gy.check("cached forward output")
